@@ -169,6 +169,45 @@ struct dfacc {
   __device__ __forceinline__ double value() const { return (double)s + (double)c; }
 };
 
+// Warp sums of 16 values at once by recursive halving: at each of four
+// exchanges a lane hands half of its values to its partner and adds the
+// partner's half to the rest, so 16 additions (and a last one) per lane do
+// what 80 would as 16 separate butterflies.  Afterwards a[0] of lane 2 q
+// holds the sum of value q (odd lanes hold it too, with the last rounding
+// taken in the other order; read the even ones).  Fixed order: deterministic.
+__device__ __forceinline__ void warp_sum16(double (&a)[16]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int h = 8, o = 16; h >= 1; h >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      const double give = up ? a[k] : a[k + h], keep = up ? a[k + h] : a[k];
+      a[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
+}
+__device__ __forceinline__ void warp_sum16(dfacc (&a)[16]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int h = 8, o = 16; h >= 1; h >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      const dfacc give = up ? a[k] : a[k + h];
+      dfacc keep = up ? a[k + h] : a[k];
+      const float s2 = __shfl_xor_sync(0xffffffffu, give.s, o);
+      const float c2 = __shfl_xor_sync(0xffffffffu, give.c, o);
+      keep.merge(s2, c2);
+      a[k] = keep;
+    }
+  }
+  const float s2 = __shfl_xor_sync(0xffffffffu, a[0].s, 1);
+  const float c2 = __shfl_xor_sync(0xffffffffu, a[0].c, 1);
+  a[0].merge(s2, c2);
+}
+
 // Host / FP64 conversions (used at set-up and output only).
 __host__ __device__ __forceinline__ dfloat df_from_double(double x) {
   const float h = (float)x;

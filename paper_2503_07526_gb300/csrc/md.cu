@@ -66,6 +66,19 @@ constexpr int kMaxRedBlocks = 152 * 64;  // reduction CTAs per replica at most
 // 0.1169; smaller CTAs lose more to the per-CTA merge and the last CTA's pass
 // (0.123 / 0.134 / 0.160 ms for 2,048 / 1,024 / 512 atoms)
 constexpr int kRedAtomsMixed = 3584;
+// Smaller replicas get smaller CTAs, a whole number of atoms per thread, down
+// to one: at 3,584 (FP64: 4,096) atoms per CTA a 4,000-atom box ran its sums
+// on one or two CTAs, a serial chain of 14 atoms per thread (34 us of an 81 us
+// step; 75 us in FP64).  With the scalar pushes a warp per series the step
+// went from 81 to 59 us at 4,000 atoms, 104 to 69 us at 37,000; the 256-replica
+// batch (8,000 CTAs instead of 736) takes the same time either way.  A function
+// of the replica's size alone, so a batch sums each replica as it would alone.
+constexpr int kRedTarget = 608;  // CTAs in flight that a replica is split for (four per SM)
+int64_t red_atoms_per_cta(int64_t n, bool fp64) {
+  const int64_t even = (n + kRedTarget - 1) / kRedTarget;
+  const int64_t whole = std::max<int64_t>(1, (even + kThreads - 1) / kThreads) * kThreads;
+  return std::min<int64_t>(fp64 ? 4096 : kRedAtomsMixed, whole);
+}
 constexpr double kRClose = 1.03;  // close-pair radius of the mixed form, in sigma
 
 // Step counters shared by all replicas.
@@ -1453,7 +1466,7 @@ __global__ void __launch_bounds__(kTileThreadsMax, 3) k_pair_tile(Sys d, LJ<floa
 // arithmetic from the double-float velocity, the double-float mass and the
 // FP32 per-particle energy and virial, and summed by a compensated FP32
 // accumulator (dfacc), so the partials carry ~48 bits like FP64 sums of
-// the same inputs; the CTA merges them in double-float too (butterflies
+// the same inputs; the CTA merges them in double-float too (recursive halving
 // across each warp, then the warps in fixed order) and converts once per
 // CTA, since FP64 instructions run at a small fraction of the FP32 rate
 // (the FP64 merge took 15 % of the kernel).  The replica tree is FP64
@@ -1469,8 +1482,7 @@ __global__ void __launch_bounds__(kTileThreadsMax, 3) k_pair_tile(Sys d, LJ<floa
 template <typename TF, typename A, bool KICK>
 __global__ void __launch_bounds__(kThreads, sizeof(TF) == 4 ? 4 : 3)
     k_kick_reduce(Sys d, double hdt) {
-  __shared__ double red[kThreads / 32][kNRed];
-  __shared__ double tot[kNRed];
+  __shared__ double red[kThreads / 32][16];
   __shared__ int last;
   const TF *F = static_cast<const TF *>(d.F);
   const TF *Ep = static_cast<const TF *>(d.epot);
@@ -1562,28 +1574,24 @@ __global__ void __launch_bounds__(kThreads, sizeof(TF) == 4 ? 4 : 3)
         for (int a = 0; a < 3; ++a) acc[11 + a].add(mv[a]);
       }
     }
-    // the CTA's sums: double-float butterflies across each warp, then the
-    // warps' results merged in fixed order (FP64 only once per CTA)
-    __shared__ float2 redf[kThreads / 32][kNRed + 3];
+    // the CTA's sums: double-float across each warp (recursive halving), then
+    // the warps' results merged in fixed order (FP64 only once per CTA)
+    __shared__ float2 redf[kThreads / 32][16];
     __shared__ double totf[kNRed + 3];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    dfacc ws[16];  // quantities 1..16
 #pragma unroll
-    for (int q = 1; q < kNRed + 3; ++q) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float s2 = __shfl_xor_sync(0xffffffffu, acc[q].s, o);
-        const float c2 = __shfl_xor_sync(0xffffffffu, acc[q].c, o);
-        acc[q].merge(s2, c2);
-      }
-      if (lane == 0) redf[warp][q] = make_float2(acc[q].s, acc[q].c);
-    }
+    for (int q = 0; q < 16; ++q) ws[q] = acc[q + 1];
+    warp_sum16(ws);
+    if ((lane & 1) == 0) redf[warp][lane >> 1] = make_float2(ws[0].s, ws[0].c);
     __syncthreads();
-    if (threadIdx.x >= 1 && threadIdx.x < kNRed + 3) {
+    if (threadIdx.x < 16) {
       dfacc a;
       a.s = redf[0][threadIdx.x].x;
       a.c = redf[0][threadIdx.x].y;
+#pragma unroll
       for (int w = 1; w < kThreads / 32; ++w) a.merge(redf[w][threadIdx.x].x, redf[w][threadIdx.x].y);
-      totf[threadIdx.x] = a.value();
+      totf[threadIdx.x + 1] = a.value();
     }
     __syncthreads();
     if (threadIdx.x < kNRed) {
@@ -1648,15 +1656,12 @@ __global__ void __launch_bounds__(kThreads, sizeof(TF) == 4 ? 4 : 3)
       acc[12] += sel * vy;
       acc[13] += sel * vz;
     }
-    double part[kNRed];  // this thread's partial sums
+    double part[16];  // this thread's partial sums
 #pragma unroll
-    for (int q = 0; q < kNRed; ++q) part[q] = (double)acc[q];
+    for (int q = 0; q < 16; ++q) part[q] = q < kNRed ? (double)acc[q] : 0.0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < kNRed; ++q) {
-      const double sm = warp_sum(part[q]);
-      if (lane == 0) red[warp][q] = sm;
-    }
+    warp_sum16(part);
+    if ((lane & 1) == 0) red[warp][lane >> 1] = part[0];
     __syncthreads();
     if (threadIdx.x < kNRed) {
       double sm = 0.0;
@@ -1674,42 +1679,46 @@ __global__ void __launch_bounds__(kThreads, sizeof(TF) == 4 ? 4 : 3)
   // the replica's partials: thread t sums CTAs t, t + 256, ... (all kNRed
   // values at once, independent loads), then a fixed tree over the threads
   {
-    double ps[kNRed];
+    double ps[16];
 #pragma unroll
-    for (int q = 0; q < kNRed; ++q) ps[q] = 0.0;
+    for (int q = 0; q < 16; ++q) ps[q] = 0.0;
     for (int b = threadIdx.x; b < R.nblk; b += kThreads) {
       const double *pp = d.partials + (R.block0 + b) * kNRed;
 #pragma unroll
       for (int q = 0; q < kNRed; ++q) ps[q] += __ldcg(pp + q);
     }
-#pragma unroll
-    for (int q = 0; q < kNRed; ++q) {
-      const double sm = warp_sum(ps[q]);
-      if (lane == 0) red[warp][q] = sm;
-    }
-    __syncthreads();
-    if (threadIdx.x < kNRed) {
-      double sm = 0.0;
-      for (int w = 0; w < kThreads / 32; ++w) sm += red[w][threadIdx.x];
-      tot[threadIdx.x] = sm;
-    }
+    warp_sum16(ps);
+    if ((lane & 1) == 0) red[warp][lane >> 1] = ps[0];
   }
   __syncthreads();
-  const int64_t nr = R.atom1 - R.atom0;
-  const double V = R.L * R.L * R.L;
-  if (threadIdx.x == 0) {
+  // one thread per observable (an FP64 division each, beside one another)
+  if (threadIdx.x < kNRed) {
+    const int q = threadIdx.x;
+    double sm = 0.0;
+    for (int w = 0; w < kThreads / 32; ++w) sm += red[w][q];
+    const int64_t nr = R.atom1 - R.atom0;
     ObsDev *ow = d.obs + r;
-    ow->K = tot[0];
-    ow->U = tot[1];
-    ow->T = nr > 1 ? 2.0 * tot[0] / (3.0 * (double)nr - 3.0) : 0.0;
-    for (int a = 0; a < 6; ++a) ow->sigma[a] = tot[2 + a] / V;
-    for (int a = 0; a < 3; ++a) ow->q[a] = tot[8 + a] / V;
-    for (int a = 0; a < 3; ++a) ow->j[a] = tot[11 + a] / V;
-    if (KICK) {
-      ow->Tsum += ow->T;
-      ow->Tn += 1;
+    if (q == 0) {
+      const double T = nr > 1 ? 2.0 * sm / (3.0 * (double)nr - 3.0) : 0.0;
+      ow->K = sm;
+      ow->T = T;
+      if (KICK) {
+        ow->Tsum += T;
+        ow->Tn += 1;
+      }
+      d.counter[r] = 0u;
+    } else if (q == 1) {
+      ow->U = sm;
+    } else {
+      const double v = sm / (R.L * R.L * R.L);
+      if (q < 8)
+        ow->sigma[q - 2] = v;
+      else if (q < 11)
+        ow->q[q - 8] = v;
+      else
+        ow->j[q - 11] = v;
     }
-    d.counter[r] = 0u;
+    __threadfence();
   }
   // the last replica to finish closes the step
   __syncthreads();
@@ -1726,26 +1735,27 @@ __global__ void __launch_bounds__(kThreads, sizeof(TF) == 4 ? 4 : 3)
   }
 }
 
-// The step's samples of the scalar correlators (Algorithm 1), one thread per
+// The step's samples of the scalar correlators (Algorithm 1), one warp per
 // series: replica r's stress series 3r..3r+2 (sigma_xy, sigma_xz, sigma_yz),
 // heat-flux series 3r..3r+2 (q_x, q_y, q_z) and mass-flux cross series
 // 6r..6r+5 ((q_a, j_a), then (j_a, j_a)), from the observables k_kick_reduce
 // wrote for the step it counted.
 __global__ void k_push_scalars(Sys d, CorrDev cs, int64_t us, CorrDev ch, int64_t uh, CorrDev cm, int64_t um) {
-  const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (k >= (int64_t)d.nrep * 12) return;
-  const int r = (int)(k / 12), tid = (int)(k % 12);
+  const int64_t k = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int per = um > 0 ? 12 : 6;
+  if (k >= (int64_t)d.nrep * per) return;
+  const int r = (int)(k / per), tid = (int)(k % per);
   const ObsDev &o = d.obs[r];
   const int64_t tc = d.st->step - d.st->corr_base;
   if (tid < 3) {
-    if (us > 0 && cs.b > 0 && tc % us == 0) push_one_series<double>(cs, 3 * r + tid, o.sigma[3 + tid], o.sigma[3 + tid], tc / us);
+    if (us > 0 && cs.b > 0 && tc % us == 0) push_series_warp<double>(cs, 3 * r + tid, o.sigma[3 + tid], o.sigma[3 + tid], tc / us);
   } else if (tid < 6) {
-    if (uh > 0 && ch.b > 0 && tc % uh == 0) push_one_series<double>(ch, 3 * r + tid - 3, o.q[tid - 3], o.q[tid - 3], tc / uh);
+    if (uh > 0 && ch.b > 0 && tc % uh == 0) push_series_warp<double>(ch, 3 * r + tid - 3, o.q[tid - 3], o.q[tid - 3], tc / uh);
   } else if (um > 0 && cm.b > 0 && tc % um == 0) {
     const int a = (tid - 6) % 3;
     const double y = o.j[a];
     const double x = tid < 9 ? o.q[a] : y;
-    push_one_series<double>(cm, 6 * r + tid - 6, x, y, tc / um);
+    push_series_warp<double>(cm, 6 * r + tid - 6, x, y, tc / um);
   }
 }
 
@@ -2332,7 +2342,7 @@ int launch_push_scalars(md_handle *h, cudaStream_t s) {
   CorrDev cs = h->bank_on[0] ? h->banks[0].c.dev : CorrDev{};
   CorrDev ch = h->bank_on[1] ? h->banks[1].c.dev : CorrDev{};
   CorrDev cm = h->bank_on[3] ? h->banks[3].c.dev : CorrDev{};
-  const int64_t threads = (int64_t)h->nrep * 12;
+  const int64_t threads = (int64_t)h->nrep * (h->bank_on[3] ? 12 : 6) * 32;  // a warp per series
   k_push_scalars<<<(int)ceil_div(threads, 128), 128, 0, s>>>(
       h->d, cs, h->bank_on[0] ? h->prm.stress.u : 0, ch, h->bank_on[1] ? h->prm.heatflux.u : 0, cm,
       h->bank_on[3] ? h->prm.massflux.u : 0);
@@ -2941,7 +2951,7 @@ int init_impl(md_handle *h, const md_params *p, const md_replica *reps, int coun
     R.atom1 = n + reps[k].n;
     R.cell0 = ncell;
     R.block0 = blocks;
-    const int64_t per_cta = h->fp64 ? 4096 : kRedAtomsMixed;
+    const int64_t per_cta = red_atoms_per_cta(reps[k].n, h->fp64);
     R.nblk = (int)std::max<int64_t>(1, std::min<int64_t>(kMaxRedBlocks, (reps[k].n + per_cta - 1) / per_cta));
     n += reps[k].n;
     ncell += (int64_t)R.nc * R.nc * R.nc;
