@@ -141,6 +141,10 @@ struct Sys {
   double *r, *v;             // FP64 form: absolute positions, velocities [3][n]
   float4 *rlo;               // mixed form: offset low words (x, y, z, 0) [n]
   float *vh, *vl;            // mixed form: velocity words [3][n]
+  float4 *relf;              // FP64 form with lists: FP32 offsets from the cell centre in units of rc (x, y, z, 0)
+  double inv_rc;             // 1 / rc, the scale of relf
+  float cut_hi;              // r^2 / rc^2 above this in FP32: outside the cutoff (see fp32_band)
+  float list_lo, list_hi;    // r^2 / rc^2 below / above these in FP32: inside / outside the list radius
   void *F, *epot, *W;        // [3][n], [n], [6][n] in the pair type
   void *rel, *relb;          // Vec4 of the pair type: current / at last rebuild
   void *vbuf;                // [vacf_slots][3][n] velocities in atom-id order, one slot per waiting
@@ -207,6 +211,10 @@ __device__ __forceinline__ void request_all(const Sys &d) {
     for (int k = threadIdx.x; k <= d.nrep; k += blockDim.x) d.rebuild[k] = 1;
 }
 
+__device__ __forceinline__ float4 scaled_rel(const Sys &d, double x, double y, double z) {
+  return make_float4((float)(x * d.inv_rc), (float)(y * d.inv_rc), (float)(z * d.inv_rc), 0.f);
+}
+
 __global__ void __launch_bounds__(kThreads) k_kick_drift64(Sys d, double hdt) {
   request_all(d);
   const double *F = static_cast<const double *>(d.F);
@@ -242,6 +250,7 @@ __global__ void __launch_bounds__(kThreads) k_kick_drift64(Sys d, double hdt) {
     const double py = fma(-(cy + 0.5), edge, x[1]);
     const double pz = fma(-(cz + 0.5), edge, x[2]);
     Vec4<double>::store(rel + i, px, py, pz, qw);
+    if (d.relf) d.relf[i] = scaled_rel(d, px, py, pz);
     const double dx = px - b.x, dy = py - b.y, dz = pz - b.z;
     if ((dx * dx + dy * dy + dz * dz) > d.lim2) request_rebuild(d, d.rep_of_atom[i]);
     bad |= !(isfinite(x[0]) && isfinite(x[1]) && isfinite(x[2]));
@@ -512,6 +521,7 @@ __global__ void __launch_bounds__(kCellWarps * 32) k_rb_rank(Sys d) {
           const double qc = d.charge[min(max(d.typeB[a], 0), 7)];
           Vec4<double>::store(static_cast<dvec4 *>(d.rel) + dst, px, py, pz, qc);
           Vec4<double>::store(static_cast<dvec4 *>(d.relb) + dst, px, py, pz, qc);
+          if (d.relf) d.relf[dst] = scaled_rel(d, px, py, pz);
         } else {
           const float *oB = reinterpret_cast<const float *>(d.rB);
           const float *wB = reinterpret_cast<const float *>(d.vB);
@@ -732,6 +742,25 @@ __global__ void __launch_bounds__(kCellWarps * 32) k_cells(Sys d, LJ<TF> lj) {
   }
 }
 
+// How far r^2 / rc^2 formed in FP32 from relf can be from the true value, for
+// values of order one: each coordinate (at most m = (1.5 edge + skin / 2) / rc
+// in magnitude) takes at most five roundings of relative size 2^-24 (two
+// conversions, the image offset's and its sum's, the difference's), so each
+// difference is off by at most 5 m 2^-24, the squared distance by at most
+// 2 sqrt(3) times that (for r near rc), and its own sum by 4 2^-24.  Doubled.
+double fp32_band(double edge, double skin, double rc) {
+  const double m = (1.5 * edge + 0.5 * skin) / rc;
+  return 2.0 * (2.0 * 1.7320508075688772 * 5.0 * m + 4.0) / 16777216.0;
+}
+
+// The FP64 form's list test of one pair: j moved into i's cell frame.
+__device__ __noinline__ bool list_test64(const dvec4 *rel, double rlist2, double edge, int i, int j, int ox, int oy,
+                                         int oz) {
+  const dvec4 pi = rel[i], pj = rel[j];
+  const double dx = pi.x - (pj.x + ox * edge), dy = pi.y - (pj.y + oy * edge), dz = pi.z - (pj.z + oz * edge);
+  return i != j && dx * dx + dy * dy + dz * dz < rlist2;
+}
+
 // Verlet-list build, one warp per chunk of 32 consecutive atoms of the
 // cell-sorted order; the lists of a chunk fill one block of maxnb rows x 32
 // lanes (slot k of atom i at block(i / 32) + 32 k + i % 32), so the pair
@@ -743,20 +772,28 @@ __global__ void __launch_bounds__(kCellWarps * 32) k_cells(Sys d, LJ<TF> lj) {
 // of the sorted order unless the row wraps), move them into the i cell's
 // frame and, for each i of the segment, test all 32 at once; a ballot and a
 // population count give every accepted j its list slot.
+//
+// FP64 form: the distance test runs in FP32 on relf, whose rounding error is
+// bounded (fp32_band), and only pairs within that band of the list radius are
+// tested again in FP64, so the lists are those of the FP64 test.  GB300's FP64
+// pipe runs at about 1/64 of its FP32 rate and the ~600 tests per atom were
+// bound by it: 397 us per build at 4,000 atoms and 1,300 at 108,000, now 127
+// and 148.
 template <typename TF, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32) k_build(Sys d, LJ<TF> lj) {
-  using V4 = typename Vec4<TF>::type;
+  using V4 = float4;
+  constexpr bool kWide = std::is_same<TF, double>::value;
   if (!any_rebuild(d)) return;
   __shared__ V4 spi[WARPS][32];
   const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
   const int64_t n = d.n;
-  const V4 *rel = static_cast<const V4 *>(d.rel);
+  const V4 *rel = kWide ? d.relf : static_cast<const V4 *>(d.rel);
   const unsigned below = (1u << lane) - 1u;
   const int64_t nchunks = (n + 31) / 32;
   for (int64_t q = blockIdx.x * (int64_t)WARPS + wl; q < nchunks; q += (int64_t)gridDim.x * WARPS) {
     const int a0 = (int)(q * 32), a1 = (int)min((int64_t)a0 + 32, n);
     __syncwarp();
-    if (a0 + lane < a1) spi[wl][lane] = Vec4<TF>::load(rel + a0 + lane);
+    if (a0 + lane < a1) spi[wl][lane] = Vec4<float>::load(rel + a0 + lane);
     __syncwarp();
     uint32_t *blk = d.nbr + q * d.maxnb * 32;
     int cnt = 0;  // lane l: list length of atom a0 + l
@@ -765,7 +802,7 @@ __global__ void __launch_bounds__(WARPS * 32) k_build(Sys d, LJ<TF> lj) {
       // the segment: atoms of s's cell within the chunk (one replica)
       const Rep &R = rep_of(d, s);
       const int nc = R.nc;
-      const TF edge = (TF)R.edge;
+      const float edge = kWide ? (float)(R.edge * d.inv_rc) : (float)R.edge;
       int cx, cy, cz;
       unpack_cell(d.cpk[s], cx, cy, cz);
       const int e = min(d.cellstart[R.cell0 + (cz * nc + cy) * nc + cx + 1], a1);
@@ -798,9 +835,9 @@ __global__ void __launch_bounds__(WARPS * 32) k_build(Sys d, LJ<TF> lj) {
             const bool jv = j < rbnd;
             const int ox = j < b1 ? -1 : (j < b2 ? 0 : 1);
             V4 t;
-            t.x = t.y = t.z = TF(0);
+            t.x = t.y = t.z = 0.f;
             if (jv) {
-              const V4 pj = Vec4<TF>::load(rel + j);
+              const V4 pj = Vec4<float>::load(rel + j);
               t.x = pj.x + ox * edge;
               t.y = pj.y + oy * edge;
               t.z = pj.z + oz * edge;
@@ -809,9 +846,13 @@ __global__ void __launch_bounds__(WARPS * 32) k_build(Sys d, LJ<TF> lj) {
             for (int ii = s; ii < e; ++ii) {
               const int li = ii - a0;  // lane that owns atom ii
               const V4 pi = spi[wl][li];
-              const TF dx = pi.x - t.x, dy = pi.y - t.y, dz = pi.z - t.z;
-              const TF r2 = dx * dx + dy * dy + dz * dz;
-              const bool acc = jv && r2 < lj.rlist2 && j != ii;
+              const float dx = pi.x - t.x, dy = pi.y - t.y, dz = pi.z - t.z;
+              const float r2 = dx * dx + dy * dy + dz * dz;
+              bool acc = jv && r2 < (kWide ? d.list_lo : (float)lj.rlist2) && j != ii;
+              if constexpr (kWide) {
+                if (jv && r2 >= d.list_lo && r2 < d.list_hi)
+                  acc = list_test64(static_cast<const dvec4 *>(d.rel), (double)lj.rlist2, R.edge, ii, j, ox, oy, oz);
+              }
               const unsigned m = __ballot_sync(0xffffffffu, acc);
               if (m) {
                 const int base = __shfl_sync(0xffffffffu, cnt, li);
@@ -830,56 +871,186 @@ __global__ void __launch_bounds__(WARPS * 32) k_build(Sys d, LJ<TF> lj) {
 }
 
 // FP64 Verlet-list pair kernel (the comparison form and the FP64 ionic
-// path): one thread per atom (cell-sorted, so a warp's neighbours overlap
-// and their coordinates come from L1), full neighbour shell, no atomics.
-// The list is streamed with evict-first loads; the loop is unrolled by
-// kUnroll so that kUnroll index loads and then kUnroll coordinate gathers
-// are in flight before the arithmetic that needs them.
+// path), full neighbour shell, no atomics.  It is bound by the FP64 pipe (two
+// results per clock and SM), so everything that need not be FP64 is not:
+//  - eight lanes share an atom.  They test its list in FP32 (relf against
+//    cut_hi, a bound that no pair inside the cutoff exceeds), eight entries at
+//    a time, and pack the entries that pass into shared memory, so the FP64
+//    rounds below run without idle lanes for the third of a list that lies in
+//    the skin;
+//  - the atom's coordinates less each image offset sit in shared memory (one
+//    FP64 operation per displacement component, no conversions), the exact
+//    cutoff test compares bit patterns, and 1/r^2 takes three FP64 operations
+//    (rcp64).
+// The eight lanes' sums are merged by recursive halving.  Eight lanes per atom
+// also fill the GPU from a few thousand atoms on, where one thread per atom
+// left all but 32 of the SMs idle.  Per step at 4,000 / 108,000 atoms
+// (Lennard-Jones) and 1,728 ions: 127 / 668 / 1,005 us with one thread per
+// atom and every operation in FP64, 26 / 418 / 97 us so.
 constexpr int kUnroll = 4;
+constexpr int kPair64Lanes = 8;
+constexpr int kPair64Fill = 128;  // list entries tested per pass
 
-template <typename TF, int POT>
-__device__ __forceinline__ void pair_from_entry(const LJ<TF> &lj, TF edge, uint32_t ent,
-                                                const typename Vec4<TF>::type &pi,
-                                                const typename Vec4<TF>::type &pj, TF f[3], TF &e, TF w[6]) {
-  int ox, oy, oz;
-  entry_image(ent, ox, oy, oz);
-  // j moved into i's cell frame first: for a close pair across a cell face
-  // pj + o lands next to pi, so the final subtraction is exact.
-  const TF dx = pi.x - (pj.x + ox * edge);
-  const TF dy = pi.y - (pj.y + oy * edge);
-  const TF dz = pi.z - (pj.z + oz * edge);
-  const TF r2 = dx * dx + dy * dy + dz * dz;
-  if (r2 < lj.rc2) lj_accumulate<TF, POT>(lj, dx, dy, dz, r2, pi.w * pj.w, f, e, w);
+// 1/x for normal positive x: the hardware's ~20-bit approximation y, then
+// y (1 + e + e^2) with e = 1 - x y (the geometric series of 1/x = y / (1 - e)),
+// whose remainder e^3 lies below FP64 rounding.
+__device__ __forceinline__ double rcp64(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
 }
 
-template <typename TF, int POT>
-__global__ void __launch_bounds__(kMaxPairThreads) k_pair_list(Sys d, LJ<TF> lj) {
-  using V4 = typename Vec4<TF>::type;
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= d.n) return;
-  const TF edge = (TF)rep_of(d, i).edge;
-  const V4 *rel = static_cast<const V4 *>(d.rel);
-  const V4 pi = Vec4<TF>::load(rel + i);
-  TF f[3] = {0, 0, 0}, e = 0, w[6] = {0, 0, 0, 0, 0, 0};
-  const int nn = d.nnb[i];
-  const uint32_t *nb = d.nbr + (i >> 5) * d.maxnb * 32 + (i & 31);
-  int k = 0;
-  for (; k + kUnroll <= nn; k += kUnroll) {
-    uint32_t ent[kUnroll];
-#pragma unroll
-    for (int u = 0; u < kUnroll; ++u) ent[u] = __ldcs(nb + (k + u) * 32);
-    V4 pj[kUnroll];
-#pragma unroll
-    for (int u = 0; u < kUnroll; ++u) pj[u] = Vec4<TF>::load(rel + entry_atom(ent[u]));
-#pragma unroll
-    for (int u = 0; u < kUnroll; ++u) pair_from_entry<TF, POT>(lj, edge, ent[u], pi, pj[u], f, e, w);
+// One pair of the FP64 form at squared distance r2: adds its energy to e (the
+// shift left out for Lennard-Jones) and returns -U'(r)/r, for Lennard-Jones
+// divided by 6.  Zero beyond the cutoff (in = false).
+template <int POT>
+__device__ __forceinline__ double pair64_terms(const LJ<double> &lj, double r2, double qq, bool in, double &e) {
+  if constexpr (POT == kPotLJ) {
+    const double ir2 = in ? rcp64(r2) : 0.0;
+    const double ir6 = ir2 * ir2 * ir2;
+    const double t = lj.c12 * ir6 * ir6;
+    const double u = fma(-lj.c6, ir6, t);  // c12 / r^12 - c6 / r^6
+    e += u;
+    return ir2 * (t + u);  // (12 c12 / r^12 - 6 c6 / r^6) / (6 r^2)
+  } else {
+    // Buckingham and the real-space Ewald term as in pair_terms, with one
+    // exponential instead of two behind erfc(x) = exp(-x^2) erfcx(x) and the
+    // Gaussian of its derivative (the rounding of x^2 put back to first order)
+    if (!in) return 0.0;
+    const double ir = rsqrt(r2), r = r2 * ir, ir2 = ir * ir, ir6 = ir2 * ir2 * ir2;
+    const double ex = lj.A * exp(-r * lj.inv_rho);
+    const double x = lj.alpha * r, x2 = x * x;
+    double gauss = exp(-x2);
+    gauss = fma(-fma(x, x, -x2), gauss, gauss);
+    const double ec = erfcx(x) * gauss, qk = lj.ke * qq * ir;
+    e += fma(qk, ec, fma(-lj.C6, ir6, ex));
+    return fma(qk, fma(ec, ir2, lj.c2 * gauss * ir), fma(-6.0 * lj.C6, ir6 * ir2, ex * lj.inv_rho * ir));
   }
-  for (; k < nn; ++k) {
-    const uint32_t ent = __ldcs(nb + k * 32);
-    const V4 pj = Vec4<TF>::load(rel + entry_atom(ent));
-    pair_from_entry<TF, POT>(lj, edge, ent, pi, pj, f, e, w);
+}
+
+template <int POT>
+__global__ void __launch_bounds__(kMaxPairThreads) k_pair_fp64(Sys d, LJ<double> lj) {
+  __shared__ double pio[kMaxPairThreads / kPair64Lanes][3][4];  // per atom and axis: its coordinate less o edge, o = -1, 0, 1
+  __shared__ float4 offf[2][64];  // image offsets in units of rc by entry bits 0..5, of the at most two replicas of the CTA
+  __shared__ uint32_t kept[kMaxPairThreads / kPair64Lanes][kPair64Fill + kPair64Lanes];
+  const int per = blockDim.x / kPair64Lanes;  // atoms of the CTA
+  const int64_t blk0 = blockIdx.x * (int64_t)per, n = d.n;
+  const int r0 = d.rep_of_atom[blk0], r1 = d.rep_of_atom[min(blk0 + per, n) - 1];
+  for (int t = threadIdx.x; t < 128; t += blockDim.x) {
+    const int which = t >> 6, code = t & 63;
+    const double edge = d.rep[which ? r1 : r0].edge;
+    int ox, oy, oz;
+    entry_image(code, ox, oy, oz);
+    offf[which][code] = scaled_rel(d, ox * edge, oy * edge, oz * edge);
   }
-  store_pair_out<TF>(d, i, f, e, w);
+  __syncthreads();
+  const int g = threadIdx.x / kPair64Lanes, l8 = threadIdx.x % kPair64Lanes;
+  const int sh = (threadIdx.x & 31) & ~(kPair64Lanes - 1);  // first lane of the group
+  const int64_t i = blk0 + g;
+  const bool live = i < n;
+  const int64_t ic = live ? i : n - 1;
+  const int which = d.rep_of_atom[ic] == r0 ? 0 : 1;
+  const dvec4 *rel = static_cast<const dvec4 *>(d.rel);
+  const dvec4 pi = Vec4<double>::load(rel + ic);
+  const float4 fi = d.relf[ic];
+  if (l8 < 3) {
+    const double edge = d.rep[d.rep_of_atom[ic]].edge;
+    pio[g][0][l8] = pi.x - (l8 - 1) * edge;
+    pio[g][1][l8] = pi.y - (l8 - 1) * edge;
+    pio[g][2][l8] = pi.z - (l8 - 1) * edge;
+  }
+  const int nn = live ? d.nnb[ic] : 0;
+  const uint32_t *nb = d.nbr + (ic >> 5) * d.maxnb * 32 + (ic & 31);
+  const int most = __reduce_max_sync(0xffffffffu, nn);  // the warp's atoms run in step
+  uint32_t *mine = kept[g];
+  const long long rc2_bits = __double_as_longlong(lj.rc2);
+  double a[16];  // F, E, W, then zeros
+#pragma unroll
+  for (int q = 0; q < 16; ++q) a[q] = 0.0;
+  int cnt = 0, in_range = 0;
+  for (int k0 = 0; k0 < most; k0 += kPair64Fill) {
+    const int k1 = min(most, k0 + kPair64Fill);
+    for (int kb = k0; kb < k1; kb += kPair64Lanes * kUnroll) {
+      uint32_t ent[kUnroll];
+#pragma unroll
+      for (int u = 0; u < kUnroll; ++u) {
+        const int k = kb + kPair64Lanes * u + l8;
+        ent[u] = k < nn && k < k1 ? __ldg(nb + k * 32) : 0u;
+      }
+      float4 fj[kUnroll];
+#pragma unroll
+      for (int u = 0; u < kUnroll; ++u) fj[u] = d.relf[entry_atom(ent[u])];
+#pragma unroll
+      for (int u = 0; u < kUnroll; ++u) {
+        const int k = kb + kPair64Lanes * u + l8;
+        const float4 o = offf[which][ent[u] & 63u];
+        const float dx = fi.x - (fj[u].x + o.x), dy = fi.y - (fj[u].y + o.y), dz = fi.z - (fj[u].z + o.z);
+        const bool keep = k < nn && k < k1 && dx * dx + dy * dy + dz * dz < d.cut_hi;
+        const unsigned m = (__ballot_sync(0xffffffffu, keep) >> sh) & ((1u << kPair64Lanes) - 1u);
+        if (keep) mine[cnt + __popc(m & ((1u << l8) - 1u))] = ent[u];
+        cnt += __popc(m);
+      }
+    }
+    __syncwarp();
+    // whole rounds of eight; the last pass takes the remainder too
+    const bool last = k0 + kPair64Fill >= most;
+    const int take = last ? cnt : cnt & ~(kPair64Lanes - 1);
+    const int upto = __reduce_max_sync(0xffffffffu, take);
+    for (int k = l8; k - l8 < upto; k += kPair64Lanes) {
+      if (k < take) {
+        const uint32_t e = mine[k];
+        const dvec4 pj = Vec4<double>::load(rel + entry_atom(e));
+        // i moved into j's cell frame first: for a close pair across a cell
+        // face it lands next to j, so the final subtraction is exact
+        const double dx = pio[g][0][e & 3u] - pj.x, dy = pio[g][1][(e >> 2) & 3u] - pj.y,
+                     dz = pio[g][2][(e >> 4) & 3u] - pj.z;
+        const double r2 = dx * dx + dy * dy + dz * dz;
+        const bool in = __double_as_longlong(r2) < rc2_bits;  // both positive: the order of the bit patterns
+        in_range += in;
+        const double fs = pair64_terms<POT>(lj, r2, pi.w * pj.w, in, a[3]);
+        const double fx = fs * dx, fy = fs * dy, fz = fs * dz;
+        a[0] += fx;
+        a[1] += fy;
+        a[2] += fz;
+        a[4] += dx * fx;
+        a[5] += dy * fy;
+        a[6] += dz * fz;
+        a[7] += dx * fy;
+        a[8] += dx * fz;
+        a[9] += dy * fz;
+      }
+    }
+    __syncwarp();
+    const int rem = cnt - take;
+    const uint32_t e = l8 < rem ? mine[take + l8] : 0u;
+    __syncwarp();
+    if (l8 < rem) mine[l8] = e;
+    cnt = rem;
+  }
+  if constexpr (POT == kPotLJ) a[3] = fma(-lj.ushift, (double)in_range, a[3]);
+  // the group's sums: lane l8 ends with values 2 l8 and 2 l8 + 1
+#pragma unroll
+  for (int h = 8, o = 4; o >= 1; h >>= 1, o >>= 1) {
+    const bool up = (l8 & o) != 0;
+#pragma unroll
+    for (int q = 0; q < h; ++q) {
+      const double give = up ? a[q] : a[q + h], keep = up ? a[q + h] : a[q];
+      a[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  if (!live || l8 > 4) return;
+  const double fscale = POT == kPotLJ ? 6.0 : 1.0;
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    const int q = 2 * l8 + s;
+    if (q < 3)
+      static_cast<double *>(d.F)[q * n + i] = fscale * a[s];
+    else if (q == 3)
+      static_cast<double *>(d.epot)[i] = 0.5 * a[s];
+    else
+      static_cast<double *>(d.W)[(q - 4) * n + i] = 0.5 * fscale * a[s];
+  }
 }
 
 // Mixed-form Verlet-list pair kernel: one thread per atom (cell-sorted, so
@@ -2283,7 +2454,7 @@ void launch_pair_pot(const md_handle *h, cudaStream_t s) {
     if constexpr (std::is_same<TF, float>::value)
       k_pair_mixed<POT><<<ceil_div(d.n, h->pair_threads), h->pair_threads, 0, s>>>(d, lj_of<float>(h->prm));
     else
-      k_pair_list<TF, POT><<<ceil_div(d.n, h->pair_threads), h->pair_threads, 0, s>>>(d, lj_of<TF>(h->prm));
+      k_pair_fp64<POT><<<ceil_div(d.n, h->pair_threads / kPair64Lanes), h->pair_threads, 0, s>>>(d, lj_of<double>(h->prm));
   } else
     k_cells<TF, POT><<<std::min(ceil_div(d.ncell, kCellWarps), 152 * 16), kCellWarps * 32, 0, s>>>(
         d, lj_of<TF>(h->prm));
@@ -2966,6 +3137,16 @@ int init_impl(md_handle *h, const md_params *p, const md_replica *reps, int coun
   const double half_skin = 0.5 * (uses_lists(*p) ? p->skin : 0.0);
   d.lim2 = half_skin * half_skin;
   d.always_rebuild = (p->pair_mode == MD_PAIR_CELLS || p->skin <= 0.0) ? 1 : 0;
+  {
+    double edge = 0.0;
+    for (const Rep &R : h->reps) edge = std::max(edge, R.edge);
+    const double band = fp32_band(edge, p->skin, p->rc), list2 = rl * rl / (p->rc * p->rc);
+    d.inv_rc = 1.0 / p->rc;
+    d.cut_hi = (float)(1.0 + band);
+    // distances near the list radius rl: the same bound, rl / rc times as large
+    d.list_lo = (float)(list2 - band * rl / p->rc);
+    d.list_hi = (float)(list2 + band * rl / p->rc);
+  }
   d.ntypes = p->ntypes;
   for (int t = 0; t < 8; ++t) {
     d.mass[t] = t < p->ntypes ? p->mass[t] : 1.0;
@@ -3012,6 +3193,7 @@ int init_impl(md_handle *h, const md_params *p, const md_replica *reps, int coun
     if (h->fp64) {
       A.take(d.r, 3 * n * sizeof(double));
       A.take(d.v, 3 * n * sizeof(double));
+      if (p->pair_mode == MD_PAIR_VERLET) A.take(d.relf, n * sizeof(float4));
     } else {
       A.take(d.rlo, n * sizeof(float4));
       A.take(d.vh, 3 * n * sizeof(float));
