@@ -82,32 +82,64 @@ __device__ __forceinline__ void mesh_add(unsigned long long *Q, int64_t idx, int
   if (hi != 0) atomicAdd(Q + K3 + idx, (unsigned long long)hi);
 }
 
+// The mesh and how a cell row's atoms are cut into CTAs (see plan_chunks).
+struct MeshPlan {
+  int K;
+  double kl;          // K / L
+  float kl_h, kl_l;   // the same as a double-float
+  int chunk, slots;   // atoms per CTA at a time; CTAs per cell row
+  int cap;            // mesh points that the gather's shared tile holds
+  int cap_spread;     // words of the spread's shared tile (rows and planes padded, see SpreadPitch)
+};
+
 // Mesh coordinates of atom i: base mesh point and fraction per axis, from
-// the cell index and the offset from the cell centre (FP64).  The base is
-// not wrapped into [0, K) (an atom that has left its cell since the last
-// sort may sit just outside the box), so that the mesh points of one cell
-// row stay contiguous; mesh indices are wrapped where the mesh is read or
-// written.
+// the cell index and the offset from the cell centre.  The base is not wrapped
+// into [0, K) (an atom that has left its cell since the last sort may sit just
+// outside the box), so that the mesh points of one cell row stay contiguous;
+// mesh indices are wrapped where the mesh is read or written.  It is kept
+// within a box of the box, so that a non-finite coordinate (which md_step
+// reports) cannot index anything.
+//
+// Mixed form: in double-float arithmetic (~48 bits, rounded to FP32 once, like
+// the FP64 arithmetic of the other form): the cell centre in mesh units is
+// (2 c + 1) K / (2 nc), split exactly into integer and fraction.  Its ~36 FP64
+// operations per atom took 33 us of each kernel at 512,000 ions.
 template <typename T>
-__device__ __forceinline__ void mesh_coords(const SpmeAtoms &a, int64_t i, double kl, int K,
+__device__ __forceinline__ void mesh_coords(const SpmeAtoms &a, int64_t i, const MeshPlan &g,
                                             const typename Rec<T>::type &r, int (&base)[3], T (&frac)[3]) {
   const int c = a.cpk[i];
   const int cc[3] = {c & 1023, (c >> 10) & 1023, c >> 20};
-  const double off[3] = {(double)r.x, (double)r.y, (double)r.z};
-  float lo[3] = {0.f, 0.f, 0.f};
-  if constexpr (std::is_same<T, float>::value) {
+  if constexpr (std::is_same<T, double>::value) {
+    const double off[3] = {r.x, r.y, r.z};
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+      const double u = ((cc[ax] + 0.5) * a.edge + off[ax]) * g.kl;
+      const double b = floor(u);
+      base[ax] = (int)b;
+      frac[ax] = u - b;
+    }
+  } else {
     const float4 l4 = a.rlo[i];
-    lo[0] = l4.x, lo[1] = l4.y, lo[2] = l4.z;
+    const float oh[3] = {r.x, r.y, r.z}, ol[3] = {l4.x, l4.y, l4.z};
+    const int den = 2 * a.nc;
+    const float fd = (float)den;
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+      const int num = (2 * cc[ax] + 1) * g.K, q = num / den;
+      const float rem = (float)(num - q * den);  // below 2^11: exact
+      const float h = rem / fd;
+      const dfloat u = df_add(dfloat{h, fmaf(-h, fd, rem) / fd}, df_mul(dfloat{oh[ax], ol[ax]}, dfloat{g.kl_h, g.kl_l}));
+      float fl = floorf(u.h), f = (u.h - fl) + u.l;
+      if (f < 0.f) {
+        f += 1.f;
+        fl -= 1.f;
+      }
+      base[ax] = q + (int)fl;
+      frac[ax] = f;
+    }
   }
 #pragma unroll
-  for (int ax = 0; ax < 3; ++ax) {
-    double x = (cc[ax] + 0.5) * a.edge + off[ax];
-    if constexpr (std::is_same<T, float>::value) x += (double)lo[ax];
-    const double u = x * kl;
-    const int b = (int)floor(u);
-    base[ax] = b;
-    frac[ax] = (T)(u - b);
-  }
+  for (int ax = 0; ax < 3; ++ax) base[ax] = max(-g.K, min(2 * g.K, base[ax]));
 }
 
 // Cardinal B-spline weights m[t] = M_N(w + t), t = 0..N-1, by the
@@ -163,11 +195,14 @@ __device__ __forceinline__ int wrap_near(int v, int K) {
   return (unsigned)w < (unsigned)K ? w : wrap(v, K);
 }
 
-constexpr int kRowThreads = 128;       // atoms per tile (one CTA)
-constexpr int kTileBytes = 48 * 1024;  // shared mesh tile of the gather
-constexpr int kSpreadTileBytes = 32 * 1024;  // shared mesh tile of the spread
-constexpr int kChunkSlots = 8;         // CTAs per cell row (each takes every 8th chunk)
-constexpr int kLoBits = 20;            // tile sums: fixed-point value = (hi << 20) + lo
+constexpr int kRowThreads = 128;       // threads of a spread or gather CTA, and the largest chunk
+constexpr int kRowWarps = kRowThreads / 32;
+constexpr int kMaxOrder = 8;
+constexpr int kSpreadPitch = 3 * kMaxOrder + 1;     // an atom's weights in the spread (odd: no bank conflicts)
+constexpr int kGatherPitch = 9 * kMaxOrder + 1;     // an atom's weights and derivatives in the gather
+constexpr int kGatherBatch = 8;                     // atoms whose weights a warp of the gather holds
+constexpr size_t kMaxTileBytes = 160 * 1024;        // shared memory that a mesh tile may take
+constexpr int kMaxTileSide = 128;                   // largest tile side in mesh points
 
 template <typename T>
 struct Two;
@@ -180,13 +215,10 @@ struct Two<double> {
   using type = double2;
 };
 
-// The mesh points of an atom: (base - t0, base - t1, base - t2) for
-// t = 0..N-1.  TILE: into a shared box of (ex, ey, ez) points whose corner
-// is mesh point (ox, oy, oz) (unwrapped); otherwise into the wrapped global
-// mesh.
-template <typename T, int N, bool TILE>
-__device__ __forceinline__ void spread_atom(const int (&base)[3], const T (&frac)[3], T q, unsigned long long *dst,
-                                            int *hi, int *lo, int K, int ox, int oy, int oz, int ey, int ez) {
+// The charge of one atom straight into the wrapped global mesh, at points
+// (base - t0, base - t1, base - t2) for t = 0..N-1.
+template <typename T, int N>
+__device__ void spread_atom(const int (&base)[3], const T (&frac)[3], T q, unsigned long long *dst, int K) {
   const int64_t K3 = (int64_t)K * K * K;
   T wx[N], wy[N], wz[N], d1[N], d2[N];
   spline<T, N, false>(frac[0], wx, d1, d2);
@@ -194,26 +226,16 @@ __device__ __forceinline__ void spread_atom(const int (&base)[3], const T (&frac
   spline<T, N, false>(frac[2], wz, d1, d2);
   int iz[N];
 #pragma unroll
-  for (int t = 0; t < N; ++t) iz[t] = TILE ? base[2] - t - oz : wrap_near(base[2] - t, K);
+  for (int t = 0; t < N; ++t) iz[t] = wrap_near(base[2] - t, K);
   for (int t0 = 0; t0 < N; ++t0) {
-    const int ix = TILE ? base[0] - t0 - ox : wrap_near(base[0] - t0, K);
+    const int ix = wrap_near(base[0] - t0, K);
     const T qx = q * wx[t0];
     for (int t1 = 0; t1 < N; ++t1) {
-      const int iy = TILE ? base[1] - t1 - oy : wrap_near(base[1] - t1, K);
+      const int iy = wrap_near(base[1] - t1, K);
       const T qxy = qx * wy[t1];
-      const int64_t row = TILE ? ((int64_t)ix * ey + iy) * ez : ((int64_t)ix * K + iy) * K;
+      const int64_t row = ((int64_t)ix * K + iy) * K;
 #pragma unroll
-      for (int t2 = 0; t2 < N; ++t2) {
-        if (TILE) {
-          // two native 32-bit shared adds: the high part (arithmetic shift)
-          // and the low 20 bits; neither can overflow over one chunk
-          const long long v = to_fix((float)(qxy * wz[t2]));
-          atomicAdd(hi + row + iz[t2], (int)(v >> kLoBits));
-          atomicAdd(lo + row + iz[t2], (int)(v & ((1ll << kLoBits) - 1)));
-        } else {
-          mesh_add(dst, row + iz[t2], K3, qxy * wz[t2]);
-        }
-      }
+      for (int t2 = 0; t2 < N; ++t2) mesh_add(dst, row + iz[t2], K3, qxy * wz[t2]);
     }
   }
 }
@@ -223,6 +245,7 @@ __device__ __forceinline__ void spread_atom(const int (&base)[3], const T (&frac
 struct Tile {
   int ox, oy, oz, ex, ey, ez;
   __device__ int64_t vol() const { return (int64_t)ex * ey * ez; }
+  __device__ bool fits(int cap) const { return vol() <= cap && max(ex, max(ey, ez)) <= kMaxTileSide; }
 };
 template <int N>
 __device__ __forceinline__ Tile chunk_tile(const int (&base)[3], bool live, int *bmin, int *bmax) {
@@ -231,12 +254,15 @@ __device__ __forceinline__ Tile chunk_tile(const int (&base)[3], bool live, int 
     bmax[threadIdx.x] = -0x7fffffff;
   }
   __syncthreads();
-  if (live)
 #pragma unroll
-    for (int ax = 0; ax < 3; ++ax) {
-      atomicMin(&bmin[ax], base[ax]);
-      atomicMax(&bmax[ax], base[ax]);
+  for (int ax = 0; ax < 3; ++ax) {
+    const int lo = __reduce_min_sync(0xffffffffu, live ? base[ax] : 0x7fffffff);
+    const int hi = __reduce_max_sync(0xffffffffu, live ? base[ax] : -0x7fffffff);
+    if ((threadIdx.x & 31) == 0) {
+      atomicMin(&bmin[ax], lo);
+      atomicMax(&bmax[ax], hi);
     }
+  }
   __syncthreads();
   Tile t;
   t.ox = bmin[0] - (N - 1);
@@ -248,86 +274,188 @@ __device__ __forceinline__ Tile chunk_tile(const int (&base)[3], bool live, int 
   return t;
 }
 
-// Charge spreading: the atoms of a cell row in chunks of kRowThreads, one
-// CTA per chunk (kChunkSlots CTAs per row).  The chunk's atoms put their bases and spline weights (q M_n in x)
-// in shared memory; the chunk's tile of mesh points is then summed column
-// by column (x, y fixed, z running), each column by one thread in the
-// order of the atoms, so no atomic is needed inside the tile and the sums
-// do not depend on scheduling; the tile's non-zero points go to the global
-// mesh in 64-bit fixed point (integer atomics: order-independent).  A chunk
-// whose tile does not fit (its atoms straddle the box edge) spreads atom by
-// atom straight into the global mesh.
+// Mesh offset of every plane, row and point of a tile (wrapped into the box),
+// so that a tile point's mesh index is three table reads and two additions.
+struct TileTable {
+  int x[kMaxTileSide], y[kMaxTileSide], z[kMaxTileSide];
+};
+__device__ __forceinline__ void fill_table(TileTable &tt, const Tile &t, int K) {
+  for (int k = threadIdx.x; k < kMaxTileSide; k += kRowThreads) {
+    if (k < t.ex) tt.x[k] = wrap_near(t.ox + k, K) * K * K;
+    if (k < t.ey) tt.y[k] = wrap_near(t.oy + k, K) * K;
+    if (k < t.ez) tt.z[k] = wrap_near(t.oz + k, K);
+  }
+}
+
+// Steps an element index k = (lx * ey + ly) * ez + lz of a tile by
+// kRowThreads without dividing: consecutive threads take consecutive z.
+struct TileWalk {
+  int lx, ly, lz, dx, dy, dz;
+  __device__ explicit TileWalk(const Tile &t) {
+    dz = kRowThreads % t.ez;
+    const int qz = kRowThreads / t.ez;
+    dy = qz % t.ey;
+    dx = qz / t.ey;
+    lz = threadIdx.x % t.ez;
+    ly = (threadIdx.x / t.ez) % t.ey;
+    lx = threadIdx.x / (t.ez * t.ey);
+  }
+  __device__ __forceinline__ int mesh_index(const TileTable &tt) const { return tt.x[lx] + tt.y[ly] + tt.z[lz]; }
+  __device__ __forceinline__ void step(const Tile &t) {
+    lz += dz;
+    ly += dy;
+    lx += dx;
+    if (lz >= t.ez) {
+      lz -= t.ez;
+      ++ly;
+    }
+    if (ly >= t.ey) {
+      ly -= t.ey;
+      ++lx;
+    }
+  }
+};
+
+// Copies one value to shared memory without holding a register for it.
+__device__ __forceinline__ void copy_async(float *dst, const float *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void copy_async(double *dst, const double *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// Row pitch and plane size of the spread's tile.  A warp adds 8 z points of two
+// neighbouring rows in two planes four apart: with the pitch a multiple of 8
+// words (not of 32) and the plane padded so that four planes lie a quarter or
+// half of the 32 banks further, its four runs of eight words fill the banks
+// once, wherever they start.
+struct SpreadPitch {
+  int row, plane;
+  __host__ __device__ SpreadPitch(int ey, int ez) {
+    row = (ez + 7) & ~7;
+    if (row % 32 == 0) row += 8;
+    plane = ey * row;  // a multiple of 8
+    plane += row % 32 == 16 ? 2 : 4;
+  }
+};
+
+// Charge spreading: the atoms of a cell row in chunks of g.chunk, one CTA per
+// chunk.  The chunk's spline weights (q M_n in x) go to shared memory, an
+// (atom, axis) pair per thread; then every warp walks all atoms and adds the
+// mesh planes it owns (those with x = its number mod 4, two of an atom's eight)
+// into the chunk's shared tile, lanes over eight z, two y and both planes.  A
+// tile point has one owner warp, which adds the atoms in order, so no atomic is
+// needed inside the tile and the sums do not depend on scheduling.  The tile's
+// non-zero points go to the global mesh in fixed point (integer atomics:
+// order-independent), consecutive lanes on consecutive z.  A chunk whose tile
+// does not fit spreads atom by atom straight into the global mesh.
+//
+// Against a thread per mesh column that tests every atom of the chunk (a third
+// of the tests hit, and its flush walked z in each thread): 440 -> 156 us at
+// 512,000 ions (mixed form, 128^3 mesh, order 8), 410 -> 35 us at 1,728 (FP64,
+// 32^3).  What is left is issue (62 %): ~260 warp instructions per atom, half
+// of them the tile additions, a fifth the flush.
 template <typename T, int N>
-__global__ void __launch_bounds__(kRowThreads) k_spme_spread(SpmeAtoms a, int K, double kl, unsigned long long *Qi) {
+__global__ void __launch_bounds__(kRowThreads) k_spme_spread(SpmeAtoms a, MeshPlan g, unsigned long long *Qi) {
   using R = typename Rec<T>::type;
   extern __shared__ __align__(16) unsigned char smraw[];
-  __shared__ int sb[3][kRowThreads];
-  __shared__ T sw[3][N][kRowThreads];  // q M_n(x), M_n(y), M_n(z) per atom
+  __shared__ int2 sb[kRowThreads];  // an atom's last tile point and its x plane there
+  __shared__ T sf[kRowThreads][3];
+  __shared__ T sq[kRowThreads];
   __shared__ int bmin[3], bmax[3];
+  __shared__ TileTable tt;
   T *tile = reinterpret_cast<T *>(smraw);
-  constexpr int64_t cap = kSpreadTileBytes / sizeof(T);
+  T *sw = tile + g.cap_spread;  // [chunk][kSpreadPitch]
   const R *rel = static_cast<const R *>(a.rel);
-  const int64_t nwork = (int64_t)a.nc * a.nc * kChunkSlots;
+  const int K = g.K, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t K3 = (int64_t)K * K * K;
+  const int z = lane & 7, y = (lane >> 3) & 1, u = lane >> 4;
+  const int64_t nwork = (int64_t)a.nc * a.nc * g.slots;
   for (int64_t wk = blockIdx.x; wk < nwork; wk += gridDim.x) {
-    const int row = (int)(wk / kChunkSlots), slot = (int)(wk % kChunkSlots);
+    const int row = (int)(wk / g.slots), slot = (int)(wk % g.slots);
     const int a0 = a.cellstart[(int64_t)row * a.nc], a1 = a.cellstart[(int64_t)row * a.nc + a.nc];
-    for (int c0 = a0 + slot * kRowThreads; c0 < a1; c0 += kChunkSlots * kRowThreads) {
+    for (int c0 = a0 + slot * g.chunk; c0 < a1; c0 += g.slots * g.chunk) {
+      const int na = min(g.chunk, a1 - c0);
       const int64_t i = c0 + threadIdx.x;
-      const bool live = i < a1;
-      const int na = min(kRowThreads, a1 - c0);
+      const bool live = (int)threadIdx.x < na;
       int base[3] = {0, 0, 0};
       T frac[3] = {T(0), T(0), T(0)};
       T q = T(0);
       if (live) {
         const R r = rel[i];
-        mesh_coords<T>(a, i, kl, K, r, base, frac);
+        mesh_coords<T>(a, i, g, r, base, frac);
         q = (T)r.w;
       }
       const Tile tl = chunk_tile<N>(base, live, bmin, bmax);
-      // pad the column length to an odd number of words (no bank conflicts)
-      const int ezp = tl.ez | 1;
-      if ((int64_t)tl.ex * tl.ey * ezp <= cap) {
+      const SpreadPitch sp(tl.ey, tl.ez);
+      if (tl.fits(g.cap_spread) && (int64_t)tl.ex * sp.plane <= g.cap_spread) {
         if (live) {
-          T w[3][N], d1[N], d2[N];
-          spline<T, N, false>(frac[0], w[0], d1, d2);
-          spline<T, N, false>(frac[1], w[1], d1, d2);
-          spline<T, N, false>(frac[2], w[2], d1, d2);
+          const int bx = base[0] - tl.ox;
+          sb[threadIdx.x] = make_int2(bx * sp.plane + (base[1] - tl.oy) * sp.row + (base[2] - tl.oz), bx);
 #pragma unroll
-          for (int t = 0; t < N; ++t) {
-            sw[0][t][threadIdx.x] = q * w[0][t];
-            sw[1][t][threadIdx.x] = w[1][t];
-            sw[2][t][threadIdx.x] = w[2][t];
-          }
+          for (int ax = 0; ax < 3; ++ax) sf[threadIdx.x][ax] = frac[ax];
+          sq[threadIdx.x] = q;
+        }
+        fill_table(tt, tl, K);
+        for (int k = threadIdx.x; k < tl.ex * sp.plane; k += kRowThreads) tile[k] = T(0);
+        __syncthreads();
+        for (int k = threadIdx.x; k < 3 * na; k += kRowThreads) {
+          const int ax = k / na, j = k - ax * na;
+          T w[N], d1[N], d2[N];
+          spline<T, N, false>(sf[j][ax], w, d1, d2);
+          const T f = ax == 0 ? sq[j] : T(1);
+          T *o = sw + j * kSpreadPitch + ax * kMaxOrder;
 #pragma unroll
-          for (int ax = 0; ax < 3; ++ax) sb[ax][threadIdx.x] = base[ax];
+          for (int t = 0; t < N; ++t) o[t] = f * w[t];
         }
         __syncthreads();
-        const int ncol = tl.ex * tl.ey;
-        for (int col = threadIdx.x; col < ncol; col += kRowThreads) {
-          const int lx = col / tl.ey, ly = col % tl.ey;
-          T *cz = tile + (int64_t)col * ezp;
-          for (int z = 0; z < tl.ez; ++z) cz[z] = T(0);
-          const int gx = tl.ox + lx, gy = tl.oy + ly;
-          for (int j = 0; j < na; ++j) {
-            const int tx = sb[0][j] - gx, ty = sb[1][j] - gy;
-            if (tx < 0 || tx >= N || ty < 0 || ty >= N) continue;
-            const T c = sw[0][tx][j] * sw[1][ty][j];
-            T *zz = cz + (sb[2][j] - tl.oz);
+        constexpr int V = N / 2;  // rows per lane
+        // the lane's point of an atom, once its last tile point is added
+        T *mine = tile - (z < N ? z : 0) - y * sp.row - u * 4 * sp.plane;
+        // the next atom's record and weights are read ahead of this one's
+        // stores, which the compiler must assume to overlap them
+        int2 b;
+        T wz, qx, wy[V];
+        auto read = [&](int j) {
+          const T *wl = sw + j * kSpreadPitch;
+          b = sb[j];
+          b.y = (b.y - warp) & 3;  // the first of this warp's planes
+          b.x -= b.y * sp.plane;
+          wz = wl[2 * kMaxOrder + (z < N ? z : 0)];
+          qx = wl[min(b.y + 4 * u, kMaxOrder - 1)];
 #pragma unroll
-            for (int t = 0; t < N; ++t) zz[-t] += c * sw[2][t][j];
+          for (int v = 0; v < V; ++v) wy[v] = wl[kMaxOrder + y + 2 * v];
+        };
+        read(0);
+        for (int j = 0; j < na; ++j) {
+          T *p = mine + b.x;
+          const bool on = z < N && b.y + 4 * u < N;
+          const T qz = qx * wz;
+          T add[V];
+#pragma unroll
+          for (int v = 0; v < V; ++v) add[v] = qz * wy[v];
+          read(min(j + 1, na - 1));
+          if (on) {
+            T t[V];
+#pragma unroll
+            for (int v = 0; v < V; ++v) t[v] = p[-2 * v * sp.row];
+#pragma unroll
+            for (int v = 0; v < V; ++v) p[-2 * v * sp.row] = t[v] + add[v];
           }
+          __syncwarp();  // the next atom's points may be other lanes'
         }
         __syncthreads();
-        for (int col = threadIdx.x; col < ncol; col += kRowThreads) {
-          const int lx = col / tl.ey, ly = col % tl.ey;
-          const int64_t g0 = ((int64_t)wrap_near(tl.ox + lx, K) * K + wrap_near(tl.oy + ly, K)) * K;
-          const T *cz = tile + (int64_t)col * ezp;
-          for (int z = 0; z < tl.ez; ++z) mesh_add(Qi, g0 + wrap_near(tl.oz + z, K), (int64_t)K * K * K, cz[z]);
-        }
+        TileWalk tw(tl);
+        const int vol = (int)tl.vol();
+        for (int k = threadIdx.x; k < vol; k += kRowThreads, tw.step(tl))
+          mesh_add(Qi, tw.mesh_index(tt), K3, tile[tw.lx * sp.plane + tw.ly * sp.row + tw.lz]);
       } else if (live) {
-        spread_atom<T, N, false>(base, frac, q, Qi, nullptr, nullptr, K, 0, 0, 0, 0, 0);
+        spread_atom<T, N>(base, frac, q, Qi, K);
       }
-      __syncthreads();  // the tile, the atom table and the extremes are reused by the next chunk
+      __syncthreads();  // the tile, the atom tables and the extremes are reused by the next chunk
     }
   }
 }
@@ -376,135 +504,227 @@ __global__ void k_spme_conv(typename Cplx<T>::type *G1, typename Cplx<T>::type *
   }
 }
 
-// The sums of one atom over its mesh points: energy (phi), force (first
-// derivatives, phi) and the six virial sums (second derivatives, psi).
-template <typename T, int N, bool TILE>
-__device__ __forceinline__ void gather_atom(const int (&base)[3], const T (&frac)[3], const T *phi, const T *psi,
-                                            const typename Two<T>::type *tile, int K, int ox, int oy, int oz, int ey,
-                                            int ez, T (&acc)[10]) {
-  T w0[N], w1[N], w2[N], d0[N], d1[N], d2[N], e0[N], e1[N], e2[N];
-  spline<T, N, true>(frac[0], w0, d0, e0);
-  spline<T, N, true>(frac[1], w1, d1, e1);
-  spline<T, N, true>(frac[2], w2, d2, e2);
-  int iz[N];
-#pragma unroll
-  for (int t = 0; t < N; ++t) iz[t] = TILE ? base[2] - t - oz : wrap_near(base[2] - t, K);
-#pragma unroll
-  for (int k = 0; k < 10; ++k) acc[k] = T(0);
-  for (int t0 = 0; t0 < N; ++t0) {
-    const int ix = TILE ? base[0] - t0 - ox : wrap_near(base[0] - t0, K);
-#pragma unroll
-    for (int t1 = 0; t1 < N; ++t1) {
-      const int iy = TILE ? base[1] - t1 - oy : wrap_near(base[1] - t1, K);
-      const int64_t row = TILE ? ((int64_t)ix * ey + iy) * ez : ((int64_t)ix * K + iy) * K;
-      const T ww = w0[t0] * w1[t1], dw = d0[t0] * w1[t1], wd = w0[t0] * d1[t1];
-      const T ew = e0[t0] * w1[t1], we = w0[t0] * e1[t1], dd = d0[t0] * d1[t1];
-#pragma unroll
-      for (int t2 = 0; t2 < N; ++t2) {
-        T p, s;
-        if (TILE) {
-          const typename Two<T>::type v = tile[row + iz[t2]];
-          p = v.x;
-          s = v.y;
-        } else {
-          p = phi[row + iz[t2]];
-          s = psi[row + iz[t2]];
-        }
-        const T pw = p * w2[t2], sw = s * w2[t2], sd = s * d2[t2];
-        acc[0] += ww * pw;
-        acc[1] += dw * pw;
-        acc[2] += wd * pw;
-        acc[3] += ww * d2[t2] * p;
-        acc[4] += ew * sw;
-        acc[5] += we * sw;
-        acc[6] += ww * e2[t2] * s;
-        acc[7] += dd * sw;
-        acc[8] += dw * sd;
-        acc[9] += wd * sd;
-      }
-    }
+// The sums of one atom over its mesh points by a group of eight lanes (lane z
+// of the group takes the points z of every (x, y)): energy (phi), force (first
+// derivatives, phi) and the six virial sums (second derivatives, psi), summed
+// axis by axis -- over x into five sums, over y into nine, then the z weights
+// give this lane's share of the ten results.  w: the atom's weights and
+// derivatives [axis][0..2][kMaxOrder].
+//
+// The (phi, psi) pairs are multiplied as pairs: two FP32 operations per
+// instruction (f32x2) in the mixed form.
+template <typename T>
+struct Pair;
+template <>
+struct Pair<float> {
+  uint64_t v;
+  __device__ __forceinline__ static Pair both(float x) {
+    Pair p;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(p.v) : "f"(x));
+    return p;
   }
+  __device__ __forceinline__ static Pair of(float2 x) {
+    Pair p;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(p.v) : "f"(x.x), "f"(x.y));
+    return p;
+  }
+  __device__ __forceinline__ void fma(Pair a, Pair b) {  // this += a b
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(v) : "l"(a.v), "l"(b.v));
+  }
+  __device__ __forceinline__ float2 get() const {
+    float2 x;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x.x), "=f"(x.y) : "l"(v));
+    return x;
+  }
+};
+template <>
+struct Pair<double> {
+  double2 v;
+  __device__ __forceinline__ static Pair both(double x) { return Pair{make_double2(x, x)}; }
+  __device__ __forceinline__ static Pair of(double2 x) { return Pair{x}; }
+  __device__ __forceinline__ void fma(Pair a, Pair b) {
+    v.x = ::fma(a.v.x, b.v.x, v.x);
+    v.y = ::fma(a.v.y, b.v.y, v.y);
+  }
+  __device__ __forceinline__ double2 get() const { return v; }
+};
+
+template <typename T, int N, typename Fetch>
+__device__ __forceinline__ void gather_lane(const T *w, int z, Fetch fetch, T (&out)[16]) {
+  using P = Pair<T>;
+  P wx[N], dx[N];
+  T ex[N];
+#pragma unroll
+  for (int t = 0; t < N; ++t) {
+    wx[t] = P::both(w[t]);
+    dx[t] = P::both(w[kMaxOrder + t]);
+    ex[t] = w[2 * kMaxOrder + t];
+  }
+  const P zero = P::both(T(0));
+  P ww = zero, dw = zero, wd = zero;  // (phi, psi): sums with weights w w, d w, w d of x and y
+  T s_ew = T(0), s_dd = T(0), s_we = T(0);
+#pragma unroll 2
+  for (int t1 = 0; t1 < N; ++t1) {
+    P c0 = zero, c1 = zero;
+    T s2 = T(0);
+#pragma unroll
+    for (int t0 = 0; t0 < N; ++t0) {
+      const typename Two<T>::type v = fetch(t0, t1);
+      const P pv = P::of(v);
+      c0.fma(wx[t0], pv);
+      c1.fma(dx[t0], pv);
+      s2 += ex[t0] * v.y;
+    }
+    const T wy = w[3 * kMaxOrder + t1], dy = w[4 * kMaxOrder + t1], ey = w[5 * kMaxOrder + t1];
+    const P wy2 = P::both(wy), dy2 = P::both(dy);
+    ww.fma(wy2, c0);
+    dw.fma(wy2, c1);
+    wd.fma(dy2, c0);
+    s_ew += wy * s2;
+    s_dd += dy * c1.get().y;
+    s_we += ey * c0.get().y;
+  }
+  const T p_ww = ww.get().x, s_ww = ww.get().y, p_dw = dw.get().x, s_dw = dw.get().y, p_wd = wd.get().x,
+          s_wd = wd.get().y;
+  const bool on = z < N;
+  const T wz = on ? w[6 * kMaxOrder + z] : T(0), dz = on ? w[7 * kMaxOrder + z] : T(0),
+          ez = on ? w[8 * kMaxOrder + z] : T(0);
+  out[0] = p_ww * wz;
+  out[1] = p_dw * wz;
+  out[2] = p_wd * wz;
+  out[3] = p_ww * dz;
+  out[4] = s_ew * wz;
+  out[5] = s_we * wz;
+  out[6] = s_ww * ez;
+  out[7] = s_dd * wz;
+  out[8] = s_dw * dz;
+  out[9] = s_wd * dz;
+#pragma unroll
+  for (int q = 10; q < 16; ++q) out[q] = T(0);
 }
 
-// Gather, one CTA per chunk of a cell row (as the spread): the chunk's tile of (phi, psi) is
-// staged in shared memory (one coalesced read per mesh point instead of one
-// per atom touching it), then every atom sums over its points.
+// Gather, one CTA per chunk of a cell row (as the spread): the chunk's tile of
+// (phi, psi) is staged in shared memory, then each warp takes eight atoms at a
+// time: 24 lanes form the weights of their three axes, and groups of eight
+// lanes sum the points of one atom each (gather_lane: 5 operations per point
+// where the separate ten sums took 14, and 64-byte rows of the tile where a
+// thread per atom read 32 unrelated places per load).  At 512,000 ions in the
+// mixed form, order 8: 297 -> 220 us; at 1,728 ions in FP64 319 -> 44 us.
 template <typename T, int N>
-__global__ void __launch_bounds__(kRowThreads, 4) k_spme_gather(SpmeAtoms a, int K, double kl, const T *phi,
-                                                             const T *psi, T ke, T kL, T cw, T self, T *F, T *epot,
-                                                             T *W) {
+__global__ void __launch_bounds__(kRowThreads, sizeof(T) == 4 ? 5 : 2)
+    k_spme_gather(SpmeAtoms a, MeshPlan g, const T *phi, const T *psi, T ke, T kL, T cw, T self, T *F, T *epot, T *W) {
   using R = typename Rec<T>::type;
   using T2 = typename Two<T>::type;
   extern __shared__ __align__(16) unsigned char smraw[];
   T2 *tile = reinterpret_cast<T2 *>(smraw);
+  T *sw = reinterpret_cast<T *>(tile + g.cap);  // [warp][kGatherBatch][kGatherPitch]
+  __shared__ TileTable tt;
+  __shared__ int sb[kRowThreads][3];
+  __shared__ T sf[kRowThreads][3];
+  __shared__ T sq[kRowThreads];
   __shared__ int bmin[3], bmax[3];
   const R *rel = static_cast<const R *>(a.rel);
   const int64_t n = a.n;
-  constexpr int64_t cap = kTileBytes / sizeof(T2);
-  const int64_t nwork = (int64_t)a.nc * a.nc * kChunkSlots;
+  const int K = g.K, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int grp = lane >> 3, z = lane & 7;
+  T *wb = sw + warp * kGatherBatch * kGatherPitch;
+  const int64_t nwork = (int64_t)a.nc * a.nc * g.slots;
   for (int64_t wk = blockIdx.x; wk < nwork; wk += gridDim.x) {
-    const int row = (int)(wk / kChunkSlots), slot = (int)(wk % kChunkSlots);
+    const int row = (int)(wk / g.slots), slot = (int)(wk % g.slots);
     const int a0 = a.cellstart[(int64_t)row * a.nc], a1 = a.cellstart[(int64_t)row * a.nc + a.nc];
-    for (int c0 = a0 + slot * kRowThreads; c0 < a1; c0 += kChunkSlots * kRowThreads) {
-      const int64_t i = c0 + threadIdx.x;
-      const bool live = i < a1;
+    for (int c0 = a0 + slot * g.chunk; c0 < a1; c0 += g.slots * g.chunk) {
+      const int na = min(g.chunk, a1 - c0);
+      const bool live = (int)threadIdx.x < na;
       int base[3] = {0, 0, 0};
       T frac[3] = {T(0), T(0), T(0)};
-      T q = T(0);
       if (live) {
-        const R r = rel[i];
-        mesh_coords<T>(a, i, kl, K, r, base, frac);
-        q = (T)r.w;
-      }
-      const Tile tl = chunk_tile<N>(base, live, bmin, bmax);
-      const bool tiled = tl.vol() <= cap;
-      if (tiled) {
-        // element k = (lx * ey + ly) * ez + lz of the tile; consecutive threads
-        // take consecutive z (coalesced), and each thread steps its (lx, ly,
-        // lz) by the mixed-radix digits of the stride instead of dividing
-        const int vol = (int)tl.vol();
-        const int dz = kRowThreads % tl.ez, qz = kRowThreads / tl.ez, dy = qz % tl.ey, dx = qz / tl.ey;
-        int lz = threadIdx.x % tl.ez, ly = (threadIdx.x / tl.ez) % tl.ey, lx = threadIdx.x / (tl.ez * tl.ey);
-        for (int k = threadIdx.x; k < vol; k += kRowThreads) {
-          const int64_t g =
-              ((int64_t)wrap_near(tl.ox + lx, K) * K + wrap_near(tl.oy + ly, K)) * K + wrap_near(tl.oz + lz, K);
-          T2 v;
-          v.x = phi[g];
-          v.y = psi[g];
-          tile[k] = v;
-          lz += dz;
-          ly += dy;
-          lx += dx;
-          if (lz >= tl.ez) {
-            lz -= tl.ez;
-            ++ly;
-          }
-          if (ly >= tl.ey) {
-            ly -= tl.ey;
-            ++lx;
-          }
+        const R r = rel[c0 + threadIdx.x];
+        mesh_coords<T>(a, c0 + threadIdx.x, g, r, base, frac);
+        sq[threadIdx.x] = (T)r.w;
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+          sb[threadIdx.x][ax] = base[ax];
+          sf[threadIdx.x][ax] = frac[ax];
         }
       }
+      const Tile tl = chunk_tile<N>(base, live, bmin, bmax);
+      const bool tiled = tl.fits(g.cap);
+      if (tiled) {
+        fill_table(tt, tl, K);
+        __syncthreads();
+        const int vol = (int)tl.vol();
+        TileWalk tw(tl);
+        for (int k = threadIdx.x; k < vol; k += kRowThreads, tw.step(tl)) {
+          const int m = tw.mesh_index(tt);
+          copy_async(&tile[k].x, phi + m);
+          copy_async(&tile[k].y, psi + m);
+        }
+        copy_async_wait();
+      }
       __syncthreads();
-      if (live) {
-        T acc[10];
-        if (tiled)
-          gather_atom<T, N, true>(base, frac, phi, psi, tile, K, tl.ox, tl.oy, tl.oz, tl.ey, tl.ez, acc);
-        else
-          gather_atom<T, N, false>(base, frac, phi, psi, tile, K, 0, 0, 0, 0, 0, acc);
-        const T er = T(0.5) * ke * q * acc[0];
-        epot[i] += er - self * q * q;
-        const T fq = -ke * q * kL;
-        F[i] += fq * acc[1];
-        F[n + i] += fq * acc[2];
-        F[2 * n + i] += fq * acc[3];
-        const T wq = cw * q;
-        W[i] += er + wq * acc[4];
-        W[n + i] += er + wq * acc[5];
-        W[2 * n + i] += er + wq * acc[6];
-        W[3 * n + i] += wq * acc[7];
-        W[4 * n + i] += wq * acc[8];
-        W[5 * n + i] += wq * acc[9];
+      for (int b0 = warp * kGatherBatch; b0 < na; b0 += kRowWarps * kGatherBatch) {
+        const int nb = min(kGatherBatch, na - b0);
+        if (lane < 3 * nb) {
+          const int j = lane / 3, ax = lane - 3 * j;
+          T m[N], d1[N], d2[N];
+          spline<T, N, true>(sf[b0 + j][ax], m, d1, d2);
+          T *o = wb + j * kGatherPitch + ax * 3 * kMaxOrder;
+#pragma unroll
+          for (int t = 0; t < N; ++t) {
+            o[t] = m[t];
+            o[kMaxOrder + t] = d1[t];
+            o[2 * kMaxOrder + t] = d2[t];
+          }
+        }
+        __syncwarp();
+        for (int h = 0; h < kGatherBatch; h += 4) {
+          if (h >= nb) break;  // uniform over the warp
+          const int j = min(h + grp, nb - 1);  // a group past the end repeats the last atom
+          const int bx = sb[b0 + j][0], by = sb[b0 + j][1], bz = sb[b0 + j][2] - min(z, N - 1);
+          // the lane's two results and what they hold now, read ahead
+          const int64_t i = c0 + b0 + j;
+          T *r0 = z == 0 ? epot + i : (z == 1 ? F + n + i : W + (2 * z - 4) * n + i);
+          T *r1 = z == 0 ? F + i : (z == 1 ? F + 2 * n + i : W + (2 * z - 3) * n + i);
+          const bool put = h + grp < nb && z < 5;
+          const T v0 = put ? *r0 : T(0), v1 = put ? *r1 : T(0);
+          T acc[16];
+          if (tiled) {
+            const int plane = tl.ey * tl.ez;
+            const T2 *p = tile + (bx - tl.ox) * plane + (by - tl.oy) * tl.ez + (bz - tl.oz);
+            gather_lane<T, N>(wb + j * kGatherPitch, z, [&](int t0, int t1) { return p[-(t0 * plane + t1 * tl.ez)]; },
+                              acc);
+          } else {
+            const int iz = wrap_near(bz, K);
+            gather_lane<T, N>(
+                wb + j * kGatherPitch, z,
+                [&](int t0, int t1) {
+                  const int64_t m = ((int64_t)wrap_near(bx - t0, K) * K + wrap_near(by - t1, K)) * K + iz;
+                  T2 v;
+                  v.x = phi[m];
+                  v.y = psi[m];
+                  return v;
+                },
+                acc);
+          }
+          // the group's sums: lane z ends with values 2 z and 2 z + 1
+#pragma unroll
+          for (int hh = 8, o = 4; o >= 1; hh >>= 1, o >>= 1) {
+            const bool up = (z & o) != 0;
+#pragma unroll
+            for (int k = 0; k < hh; ++k) {
+              const T give = up ? acc[k] : acc[k + hh], keep = up ? acc[k + hh] : acc[k];
+              acc[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+            }
+          }
+          const T q = sq[b0 + j];
+          const T er = T(0.5) * ke * q * __shfl_sync(0xffffffffu, acc[0], lane & 24);
+          if (put) {
+            const T fq = -ke * q * kL, wq = cw * q;
+            *r0 = v0 + (z == 0 ? er - self * q * q : (z == 1 ? fq * acc[0] : (z < 4 ? er : T(0)) + wq * acc[0]));
+            *r1 = v1 + (z < 2 ? fq * acc[1] : (z == 2 ? er : T(0)) + wq * acc[1]);
+          }
+        }
+        __syncwarp();  // the batch's weights are rewritten next
       }
       __syncthreads();
     }
@@ -529,6 +749,32 @@ int cufft_ok(cufftResult r, const char *what) {
 
 int grid_of(int64_t n) { return (int)std::min<int64_t>((n + 255) / 256, 152 * 16); }
 
+constexpr size_t kMaxSpmeSmem =
+    kMaxTileBytes + std::max(kRowWarps * kGatherBatch * kGatherPitch, kRowThreads * kSpreadPitch) * sizeof(double);
+static_assert(kMaxSpmeSmem + 8 * 1024 <= 227 * 1024, "tile, weights and static tables fit one CTA");
+
+// Chunk and tile sizes: the largest chunk of 128, 64 or 32 atoms that still
+// gives four CTAs per SM (128 atoms share a tile's halo: at 512,000 ions 10
+// tile points are flushed per mesh point, against 17 with 32 atoms; below
+// 78,000 atoms more CTAs count for more), whose expected tile of the gather
+// (the cells the chunk spans plus the spline's support) fits.
+void plan_chunks(const SpmeAtoms &a, int order, size_t ts, MeshPlan &g) {
+  const double cells = (double)a.nc * a.nc * a.nc, apc = a.n / cells, e = a.edge * g.kl;
+  double pts = 0.0, words = 0.0;
+  for (g.chunk = kRowThreads; g.chunk >= 32; g.chunk /= 2) {
+    const double side = std::ceil(e) + order + 1, len = std::ceil(e * std::min<double>(a.nc, g.chunk / apc + 1.0)) + order + 1;
+    const SpreadPitch sp((int)side, (int)side);
+    pts = side * side * len;
+    words = len * sp.plane;
+    if (g.chunk == 32 || (a.n >= (int64_t)608 * g.chunk && pts * 2 * ts <= kMaxTileBytes / 2)) break;
+  }
+  g.cap = (int)std::min(pts, (double)(kMaxTileBytes / (2 * ts)));
+  g.cap = (g.cap + 3) & ~3;
+  if ((size_t)g.cap * 2 * ts > kMaxTileBytes) g.cap -= 4;
+  g.cap_spread = (int)std::min(words, (double)(kMaxTileBytes / ts)) & ~3;
+  g.slots = std::max(1, (int)std::ceil(apc * a.nc / g.chunk));
+}
+
 }  // namespace
 
 int Spme::create(const SpmeParams &p, bool fp64, cudaStream_t st) {
@@ -547,10 +793,11 @@ int Spme::create(const SpmeParams &p, bool fp64, cudaStream_t st) {
   }
   OTF_CUDA(cudaMalloc(&Qi_, sizeof(unsigned long long) * K3 * (fp64 ? 2 : 1)));  // 128-bit points in FP64
   OTF_CUDA(cudaMalloc(&Qr_, ts * K3));
-  OTF_CUDA(cudaMalloc(&phi_, ts * K3));
-  OTF_CUDA(cudaMalloc(&psi_, ts * K3));
-  OTF_CUDA(cudaMalloc(&G1_, 2 * ts * KH));
-  OTF_CUDA(cudaMalloc(&G2_, 2 * ts * KH));
+  // both convolved meshes, and their spectra, end to end: one batched inverse
+  OTF_CUDA(cudaMalloc(&phi_, 2 * ts * K3));
+  psi_ = static_cast<char *>(phi_) + ts * K3;
+  OTF_CUDA(cudaMalloc(&G1_, 4 * ts * KH));
+  G2_ = static_cast<char *>(G1_) + 2 * ts * KH;
   OTF_CUDA(cudaMalloc(&bmod_, ts * K));
   if (fp64) {
     OTF_CUDA(cudaMemcpy(bmod_, bm.data(), sizeof(double) * K, cudaMemcpyHostToDevice));
@@ -559,7 +806,10 @@ int Spme::create(const SpmeParams &p, bool fp64, cudaStream_t st) {
     OTF_CUDA(cudaMemcpy(bmod_, bf.data(), sizeof(float) * K, cudaMemcpyHostToDevice));
   }
   int rc = cufft_ok(cufftPlan3d(&fwd_, K, K, K, fp64 ? CUFFT_D2Z : CUFFT_R2C), "cufftPlan3d (forward)");
-  if (!rc) rc = cufft_ok(cufftPlan3d(&inv_, K, K, K, fp64 ? CUFFT_Z2D : CUFFT_C2R), "cufftPlan3d (inverse)");
+  int dims[3] = {K, K, K};
+  if (!rc)
+    rc = cufft_ok(cufftPlanMany(&inv_, 3, dims, nullptr, 1, 0, nullptr, 1, 0, fp64 ? CUFFT_Z2D : CUFFT_C2R, 2),
+                  "cufftPlanMany (inverse)");
   if (rc) return rc;
   plans_ = true;
   rc = cufft_ok(cufftSetStream(fwd_, st), "cufftSetStream");
@@ -573,7 +823,7 @@ void Spme::destroy() {
     cufftDestroy(inv_);
     plans_ = false;
   }
-  for (void *q : {(void *)Qi_, Qr_, phi_, psi_, G1_, G2_, bmod_})
+  for (void *q : {(void *)Qi_, Qr_, phi_, G1_, bmod_})
     if (q) cudaFree(q);
   Qi_ = nullptr;
   Qr_ = phi_ = psi_ = G1_ = G2_ = bmod_ = nullptr;
@@ -593,25 +843,32 @@ int Spme::run_t(const SpmeAtoms &a, T *F, T *epot, T *W, cudaStream_t st) {
     set_error("spme: the cell list is missing");
     return MD_EINVAL;
   }
-  const int rows = (int)std::min<int64_t>((int64_t)a.nc * a.nc * kChunkSlots, 152 * 32);
+  MeshPlan g;
+  g.K = K;
+  g.kl = kl;
+  const dfloat kd = df_from_double(kl);
+  g.kl_h = kd.h;
+  g.kl_l = kd.l;
+  plan_chunks(a, p_.order, sizeof(T), g);
+  const int grid = (int)std::min<int64_t>((int64_t)a.nc * a.nc * g.slots, 152 * 64);
+  const size_t spread_smem = ((size_t)g.cap_spread + (size_t)g.chunk * kSpreadPitch) * sizeof(T);
+  const size_t gather_smem = ((size_t)2 * g.cap + (size_t)kRowWarps * kGatherBatch * kGatherPitch) * sizeof(T);
   if (!attr_) {
     for (const void *f : {(const void *)k_spme_spread<T, 4>, (const void *)k_spme_spread<T, 6>,
-                          (const void *)k_spme_spread<T, 8>})
-      OTF_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpreadTileBytes));
-    for (const void *f : {(const void *)k_spme_gather<T, 4>, (const void *)k_spme_gather<T, 6>,
-                          (const void *)k_spme_gather<T, 8>})
-      OTF_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileBytes));
+                          (const void *)k_spme_spread<T, 8>, (const void *)k_spme_gather<T, 4>,
+                          (const void *)k_spme_gather<T, 6>, (const void *)k_spme_gather<T, 8>})
+      OTF_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSpmeSmem));
     attr_ = true;
   }
   switch (p_.order) {
     case 4:
-      k_spme_spread<T, 4><<<rows, kRowThreads, kSpreadTileBytes, st>>>(a, K, kl, Qi_);
+      k_spme_spread<T, 4><<<grid, kRowThreads, spread_smem, st>>>(a, g, Qi_);
       break;
     case 6:
-      k_spme_spread<T, 6><<<rows, kRowThreads, kSpreadTileBytes, st>>>(a, K, kl, Qi_);
+      k_spme_spread<T, 6><<<grid, kRowThreads, spread_smem, st>>>(a, g, Qi_);
       break;
     default:
-      k_spme_spread<T, 8><<<rows, kRowThreads, kSpreadTileBytes, st>>>(a, K, kl, Qi_);
+      k_spme_spread<T, 8><<<grid, kRowThreads, spread_smem, st>>>(a, g, Qi_);
   }
   k_spme_unfix<T><<<grid_of(K3), 256, 0, st>>>(Qi_, static_cast<T *>(Qr_), K3);
   OTF_LAUNCH_CHECK();
@@ -629,10 +886,8 @@ int Spme::run_t(const SpmeAtoms &a, T *F, T *epot, T *W, cudaStream_t st) {
   OTF_LAUNCH_CHECK();
   if constexpr (std::is_same<T, double>::value) {
     rc = cufft_ok(cufftExecZ2D(inv_, static_cast<C *>(G1_), static_cast<double *>(phi_)), "cufftExecZ2D");
-    if (!rc) rc = cufft_ok(cufftExecZ2D(inv_, static_cast<C *>(G2_), static_cast<double *>(psi_)), "cufftExecZ2D");
   } else {
     rc = cufft_ok(cufftExecC2R(inv_, static_cast<C *>(G1_), static_cast<float *>(phi_)), "cufftExecC2R");
-    if (!rc) rc = cufft_ok(cufftExecC2R(inv_, static_cast<C *>(G2_), static_cast<float *>(psi_)), "cufftExecC2R");
   }
   if (rc) return rc;
   const T ke = (T)p_.ke, kL = (T)kl, cw = (T)(p_.ke * kl * kl / (8.0 * kPi * kPi)),
@@ -640,13 +895,13 @@ int Spme::run_t(const SpmeAtoms &a, T *F, T *epot, T *W, cudaStream_t st) {
   const T *phi = static_cast<const T *>(phi_), *psi = static_cast<const T *>(psi_);
   switch (p_.order) {
     case 4:
-      k_spme_gather<T, 4><<<rows, kRowThreads, kTileBytes, st>>>(a, K, kl, phi, psi, ke, kL, cw, self, F, epot, W);
+      k_spme_gather<T, 4><<<grid, kRowThreads, gather_smem, st>>>(a, g, phi, psi, ke, kL, cw, self, F, epot, W);
       break;
     case 6:
-      k_spme_gather<T, 6><<<rows, kRowThreads, kTileBytes, st>>>(a, K, kl, phi, psi, ke, kL, cw, self, F, epot, W);
+      k_spme_gather<T, 6><<<grid, kRowThreads, gather_smem, st>>>(a, g, phi, psi, ke, kL, cw, self, F, epot, W);
       break;
     default:
-      k_spme_gather<T, 8><<<rows, kRowThreads, kTileBytes, st>>>(a, K, kl, phi, psi, ke, kL, cw, self, F, epot, W);
+      k_spme_gather<T, 8><<<grid, kRowThreads, gather_smem, st>>>(a, g, phi, psi, ke, kL, cw, self, F, epot, W);
   }
   OTF_LAUNCH_CHECK();
   return MD_OK;

@@ -49,8 +49,8 @@ class Spme {
   bool fp64_ = false;
   unsigned long long *Qi_ = nullptr;  // fixed-point charge mesh (deterministic sums)
   void *Qr_ = nullptr;                // real mesh [K^3]
-  void *G1_ = nullptr, *G2_ = nullptr;  // half spectra [K][K][K/2+1]
-  void *phi_ = nullptr, *psi_ = nullptr;  // convolved meshes [K^3]
+  void *G1_ = nullptr, *G2_ = nullptr;  // half spectra [K][K][K/2+1], one allocation (G1_)
+  void *phi_ = nullptr, *psi_ = nullptr;  // convolved meshes [K^3], one allocation (phi_)
   void *bmod_ = nullptr;              // |b(m)|^2 [K]
   cufftHandle fwd_ = 0, inv_ = 0;
   bool plans_ = false;
