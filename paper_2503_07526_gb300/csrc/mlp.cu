@@ -773,9 +773,19 @@ struct AdamTable {
   AdamLayer l[kMaxLayers];
   int n;
 };
+struct AdamStep {
+  float lr, beta1, beta2, eps, wd, c1, c2;
+};
+// One parameter's step; decay: the weight decay of this parameter (0: a bias).
+__device__ __forceinline__ float adam_one(const AdamStep &k, float w, float g, float &m1, float &m2, bool decay) {
+  m1 = k.beta1 * m1 + (1.f - k.beta1) * g;
+  m2 = k.beta2 * m2 + (1.f - k.beta2) * g * g;
+  float step = (m1 / k.c1) / (sqrtf(m2 / k.c2) + k.eps);
+  if (decay) step += k.wd * w;
+  return w - k.lr * step;
+}
 __global__ void k_adam(float *__restrict__ w, const float *__restrict__ g, float *__restrict__ m1,
-                       float *__restrict__ m2, int64_t count, AdamTable tab, float lr, float beta1, float beta2,
-                       float eps, float wd, float c1, float c2) {
+                       float *__restrict__ m2, int64_t count, AdamTable tab, AdamStep k) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
     int L = 0;
     bool is_w = false;
@@ -787,14 +797,10 @@ __global__ void k_adam(float *__restrict__ w, const float *__restrict__ g, float
       }
       if (i >= A.b_off && i < A.b_off + A.out_p) L = l;
     }
-    const float gi = g[i];
-    const float a = beta1 * m1[i] + (1.f - beta1) * gi;
-    const float b = beta2 * m2[i] + (1.f - beta2) * gi * gi;
+    float a = m1[i], b = m2[i];
+    const float wn = adam_one(k, w[i], g[i], a, b, is_w);
     m1[i] = a;
     m2[i] = b;
-    float step = (a / c1) / (sqrtf(b / c2) + eps);
-    if (is_w) step += wd * w[i];
-    const float wn = w[i] - lr * step;
     w[i] = wn;
     if (is_w) {
       const AdamLayer &A = tab.l[L];
@@ -817,6 +823,379 @@ __global__ void k_cast_weights(const float *__restrict__ w, AdamTable tab) {
     A.wb[j] = v;
     if (A.wtb) A.wtb[(int64_t)c * A.ld_t + o] = v;
   }
+}
+
+// ------------------------------------------------- training, many steps per launch
+//
+// All the steps of an epoch in one launch of one cluster of eight CTAs.  A
+// step is a chain of small products (128 x 128 x 128 for a batch of 128) with
+// nothing to fill the GPU with, so its time is latency: as one launch of one
+// CTA per product it took 230 us (11 products of 6 to 27 us, their epilogues a
+// thread per row).  Here every product is cut into column slices over the
+// eight CTAs, and the phases of a step (one per layer forward, one per layer
+// back, the last weight gradient with Adam) are separated by cluster barriers:
+// TRAIN_FIGS per step.  Operands go through global memory (L2) in the same
+// matrices as the layered kernels use and come back by TMA, the writers
+// fencing the async proxy before each barrier; each weight gradient's product
+// runs beside the next layer's and stays in TMEM until Adam reads it there.
+// Every element's products are accumulated in the same order as in k_gemm_tc,
+// and rounding points and epilogue arithmetic are the same.
+constexpr int kTrainCtas = 8;
+constexpr int kTrainThreads = 256;
+constexpr int kTrainStages = 6;
+constexpr uint32_t kStageBytes = 2 * kPanelBytes;  // an A and a B panel of up to 128 rows
+constexpr int kGradCol = 128;                      // TMEM: layer l's gradient slices at kGradCol + 32 l
+constexpr size_t kTrainSmem = 1024 + (size_t)kTrainStages * kStageBytes;
+
+struct TrainMaps {
+  CUtensorMap x, xt;                     // this epoch's inputs: boxes of 128 rows; transposed, boxes of 16
+  CUtensorMap h[kMaxLayers], dz[kMaxLayers], dzt[kMaxLayers], dy, ht_last;  // A operands, boxes of 128 rows
+  CUtensorMap w[kMaxLayers], wt[kMaxLayers], ht[kMaxLayers], dyt;           // B operands, boxes of 16 rows
+};
+struct TrainArgs {
+  int L, n_out, cap, nb;
+  int in_k[kMaxLayers];
+  AdamTable tab;
+  AdamStep adam;             // c1, c2 come from corr
+  const float2 *corr;        // [nb] bias corrections of each step
+  float *w, *g, *m1, *m2;
+  bf16 *H[kMaxLayers], *Ht[kMaxLayers], *dZ[kMaxLayers], *dZt[kMaxLayers], *dY, *dYt;
+  const float *Ts;           // [nb cap][n_out] standardised targets in epoch order
+  double *part, *loss;       // [cap / 128] a batch's partial losses; [2] as in k_loss_dy
+  double acc_scale;
+  unsigned *err;
+  uint64_t wait_ns;
+};
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+// Global writes of this thread made visible to other CTAs' TMA loads (the
+// barrier that follows orders them; the reader fences too).
+__device__ __forceinline__ void publish() {
+  __threadfence();
+  asm volatile("fence.proxy.async;" ::: "memory");
+}
+// 8 consecutive FP32 columns of this thread's TMEM lane.
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ uint4 pack8(const bf16 (&b)[8]) {
+  uint4 q;
+  bf16 *o = reinterpret_cast<bf16 *>(&q);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) o[i] = b[i];
+  return q;
+}
+
+__global__ void __cluster_dims__(kTrainCtas, 1, 1) __launch_bounds__(kTrainThreads, 1)
+    k_train_cluster(const __grid_constant__ TrainMaps tm, const __grid_constant__ TrainArgs a) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  __shared__ uint64_t bars[2 * kTrainStages + 2];  // full[S], empty[S], product done, gradients done
+  __shared__ uint32_t slot;
+  __shared__ volatile int dead;  // a wait gave up: no more products, epilogues or updates, only the barriers
+  __shared__ double wpart[kTrainThreads / 32];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, rank = (int)blockIdx.x;
+  const int quarter = warp & 3, half = warp >> 2, row = quarter * 32 + lane;  // TMEM lane and column half
+  const uint32_t done_bar = smem_u32(&bars[2 * kTrainStages]), grad_bar = smem_u32(&bars[2 * kTrainStages + 1]);
+  if (tid == 0) {
+    for (int s = 0; s < 2 * kTrainStages + 2; ++s) mbar_init(smem_u32(&bars[s]), 1);
+    dead = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) tmem_alloc(smem_u32(&slot), 512);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = slot;
+  const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16);
+  const int L = a.L, mt = a.cap / kBM;
+  const int nsl = mt >= kTrainCtas ? 1 : kTrainCtas / mt;  // column slices of a 128-wide product
+  const int wsl = kBM / nsl, tiles = mt * nsl;
+
+  // thread 0: panels issued and consumed so far (stage = count mod kTrainStages)
+  uint32_t issued = 0, consumed = 0;
+  // D [128 x N] at TMEM column col += A rows [arow, +128) x B rows [brow, +N)
+  // over K columns from ak and bk (thread 0; two or more panels in flight)
+  auto product = [&](const CUtensorMap *ma, int arow, int ak, const CUtensorMap *mb, int brow, int bk, int K, int N,
+                     int col) {
+    if (dead) return;
+    const int np = (K + kBK - 1) / kBK;
+    const uint32_t idesc = idesc_bf16(kBM, N);
+    int in = 0;
+    for (int p = 0; p < np; ++p) {
+      for (; in < np && in < p + kTrainStages; ++in, ++issued) {
+        const uint32_t s = issued % kTrainStages, use = issued / kTrainStages;
+        if (use > 0 && !mbar_wait_for(smem_u32(&bars[kTrainStages + s]), (use - 1) & 1u, a.wait_ns)) {
+          dead = 1;
+          return;
+        }
+        const uint32_t fb = smem_u32(&bars[s]), sa = smem_u32(smem + s * kStageBytes);
+        mbar_expect_tx(fb, kPanelBytes + (uint32_t)N * 128u);
+        tma_load_2d(sa, ma, ak + in * kBK, arow, fb);
+        for (int r = 0; r < N; r += 16) tma_load_2d(sa + kPanelBytes + r * 128u, mb, bk + in * kBK, brow + r, fb);
+      }
+      const uint32_t s = consumed % kTrainStages;
+      if (!mbar_wait_for(smem_u32(&bars[s]), (consumed / kTrainStages) & 1u, a.wait_ns)) {
+        dead = 1;
+        return;
+      }
+      ++consumed;
+      tc_fence_after();
+      const uint32_t a0 = smem_u32(smem + s * kStageBytes), b0 = a0 + kPanelBytes;
+      const int nk = min(kBK, K - p * kBK) / 16;
+      for (int j = 0; j < nk; ++j)
+        mma_bf16(tmem + (uint32_t)col, sw128_desc(a0 + 32u * j), sw128_desc(b0 + 32u * j), idesc, (p | j) != 0);
+      mma_commit(smem_u32(&bars[kTrainStages + s]));
+    }
+  };
+  uint32_t phase = 0;
+  // waits for the product committed to done_bar (every thread); false: skip the epilogue
+  auto finish = [&]() {
+    const bool ok = mbar_wait(done_bar, phase);
+    phase ^= 1u;
+    if (!ok) dead = 1;
+    tc_fence_after();
+    __syncthreads();
+    const bool run = dead == 0;
+    __syncthreads();  // thread 0 may set it again in the next product
+    return run;
+  };
+
+  for (int step = 0; step < a.nb; ++step) {
+    const int row0 = step * a.cap;
+    // forward
+    for (int l = 0; l < L - 1; ++l) {
+      for (int t = rank; t < tiles; t += kTrainCtas) {
+        const int m0 = (t / nsl) * kBM, n0 = (t % nsl) * wsl;
+        if (tid == 0) {
+          asm volatile("fence.proxy.async;" ::: "memory");
+          product(l == 0 ? &tm.x : &tm.h[l - 1], (l == 0 ? row0 : 0) + m0, 0, &tm.w[l], n0, 0, a.in_k[l], wsl, 0);
+          mma_commit(done_bar);
+        }
+        if (finish()) {
+          const float *bias = a.w + a.tab.l[l].b_off + n0;
+          const int64_t m = m0 + row;
+          for (int c0 = half * (wsl / 2); c0 < (half + 1) * (wsl / 2); c0 += 8) {
+            float v[8];
+            tmem_ld8(trow + (uint32_t)c0, v);
+            bf16 b[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) b[i] = __float2bfloat16_rn(tanhf(v[i] + __ldcg(bias + c0 + i)));
+            *reinterpret_cast<uint4 *>(a.H[l] + m * kBM + n0 + c0) = pack8(b);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) a.Ht[l][(int64_t)(n0 + c0 + i) * a.cap + m] = b[i];
+          }
+        }
+        tc_fence_before();
+        __syncthreads();
+      }
+      publish();
+      cluster_sync();
+    }
+    // output layer, loss and its gradient (tile t: rows of one CTA)
+    for (int t = rank; t < mt; t += kTrainCtas) {
+      if (tid == 0) {
+        asm volatile("fence.proxy.async;" ::: "memory");
+        product(&tm.h[L - 2], t * kBM, 0, &tm.w[L - 1], 0, 0, a.in_k[L - 1], kOutPad, 0);
+        mma_commit(done_bar);
+      }
+      double acc = 0.0;
+      if (finish()) {
+        const float *bias = a.w + a.tab.l[L - 1].b_off;
+        const int64_t m = (int64_t)t * kBM + row;
+        const float gscale = (float)(2.0 * (1.0 / ((double)a.cap * a.n_out)));
+        float v[8];
+        tmem_ld8(trow + (uint32_t)(half * 8), v);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int c = half * 8 + i;
+          if (c < a.n_out) {
+            const float d = (v[i] + __ldcg(bias + c)) - a.Ts[(row0 + m) * a.n_out + c];
+            acc += (double)d * d;
+            const bf16 db = __float2bfloat16_rn(gscale * d);
+            a.dY[m * 64 + c] = db;
+            a.dYt[(int64_t)c * a.cap + m] = db;
+          }
+        }
+      }
+      acc = warp_sum(acc);
+      if (lane == 0) wpart[warp] = acc;
+      tc_fence_before();
+      __syncthreads();
+      if (tid == 0) {
+        double s = 0.0;
+        for (int w = 0; w < kTrainThreads / 32; ++w) s += wpart[w];
+        a.part[t] = s;
+      }
+    }
+    publish();
+    cluster_sync();
+    // back: dZ_l = (dZ_{l+1} W_{l+1}) (1 - H_l^2), and beside it the weight
+    // gradient of layer l + 1, left in TMEM
+    for (int l = L - 2; l >= 0; --l) {
+      const bool top = l == L - 2;
+      bool graded = false;
+      for (int t = rank; t < tiles || !graded; t += kTrainCtas) {
+        const bool mine = t < tiles;
+        const int m0 = (t / nsl) * kBM, n0 = (t % nsl) * wsl;
+        if (tid == 0) {
+          asm volatile("fence.proxy.async;" ::: "memory");
+          if (mine) {
+            product(top ? &tm.dy : &tm.dz[l + 1], m0, 0, &tm.wt[l + 1], n0, 0, top ? kOutPad : kBM, wsl, 0);
+            mma_commit(done_bar);
+          }
+          if (!graded) {
+            if (!top)
+              product(&tm.dzt[l + 1], 0, 0, &tm.ht[l], rank * 16, 0, a.cap, 16, kGradCol + 32 * (l + 1));
+            else if (rank == kTrainCtas - 1)
+              product(&tm.ht_last, 0, 0, &tm.dyt, 0, 0, a.cap, kOutPad, kGradCol + 32 * (l + 1));
+          }
+        }
+        graded = true;
+        __syncwarp();
+        if (!mine) break;
+        if (finish()) {
+          const int64_t m = m0 + row;
+          for (int c0 = half * (wsl / 2); c0 < (half + 1) * (wsl / 2); c0 += 8) {
+            float v[8];
+            tmem_ld8(trow + (uint32_t)c0, v);
+            const uint4 hq = __ldcg(reinterpret_cast<const uint4 *>(a.H[l] + m * kBM + n0 + c0));
+            const bf16 *hb = reinterpret_cast<const bf16 *>(&hq);
+            bf16 b[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const float hd = __bfloat162float(hb[i]);
+              b[i] = __float2bfloat16_rn(v[i] * (1.0f - hd * hd));
+            }
+            *reinterpret_cast<uint4 *>(a.dZ[l] + m * kBM + n0 + c0) = pack8(b);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) a.dZt[l][(int64_t)(n0 + c0 + i) * a.cap + m] = b[i];
+          }
+        }
+        tc_fence_before();
+        __syncthreads();
+      }
+      publish();
+      cluster_sync();
+    }
+    // the first layer's weight gradient, the bias gradients meanwhile, then Adam
+    const float2 corr = __ldg(a.corr + step);
+    AdamStep ad = a.adam;
+    ad.c1 = corr.x;
+    ad.c2 = corr.y;
+    const bool keep_g = step == a.nb - 1;  // the last batch's gradients stay readable, as after the layered step
+    if (tid == 0) {
+      asm volatile("fence.proxy.async;" ::: "memory");
+      for (int s = rank, k = 0; s * 16 < a.in_k[0]; s += kTrainCtas, ++k)
+        product(&tm.dzt[0], 0, 0, &tm.xt, s * 16, row0, a.cap, 16, kGradCol + 16 * k);
+      mma_commit(grad_bar);
+      if (rank == 0) {
+        double s = 0.0;
+        for (int t = 0; t < mt; ++t) s += __ldcg(a.part + t);
+        s *= 1.0 / ((double)a.cap * a.n_out);
+        a.loss[0] += s * a.acc_scale;
+        a.loss[1] = s;
+      }
+    }
+    if (warp > 0 && !dead) {
+      for (int q = rank * 7 + warp - 1; q < (L - 1) * kBM + kOutPad; q += kTrainCtas * 7) {
+        const int l = min(q / kBM, L - 1), n = q - l * kBM;
+        const bf16 *src = (l < L - 1 ? a.dZt[l] : a.dYt) + (int64_t)n * a.cap;
+        float acc = 0.f;
+        for (int m = lane; m < a.cap; m += 32)
+          acc += __bfloat162float(__ushort_as_bfloat16(__ldcg(reinterpret_cast<const unsigned short *>(src) + m)));
+        acc = warp_sum(acc);
+        if (lane == 0) {
+          const int64_t i = a.tab.l[l].b_off + n;
+          float m1 = __ldcg(a.m1 + i), m2 = __ldcg(a.m2 + i);
+          a.w[i] = adam_one(ad, __ldcg(a.w + i), acc, m1, m2, false);
+          a.m1[i] = m1;
+          a.m2[i] = m2;
+          if (keep_g) a.g[i] = acc;
+        }
+      }
+    }
+    __syncwarp();
+    const bool gok = mbar_wait(grad_bar, (uint32_t)step & 1u);
+    if (!gok) dead = 1;
+    tc_fence_after();
+    __syncthreads();
+    const bool update = dead == 0;
+    if (update) {
+      for (int l = 0; l < L - 1; ++l) {
+        const AdamLayer &A = a.tab.l[l];
+        for (int s = rank, k = 0; s * 16 < a.in_k[l]; s += kTrainCtas, ++k) {
+          float v[8];
+          tmem_ld8(trow + (uint32_t)(kGradCol + 32 * l + 16 * k + half * 8), v);
+          const int c = s * 16 + half * 8;  // eight input columns of output row `row`
+          const int64_t i = A.w_off + (int64_t)row * A.in_k + c;
+          float wv[8], m1[8], m2[8];
+#pragma unroll
+          for (int h4 = 0; h4 < 8; h4 += 4) {
+            *reinterpret_cast<float4 *>(wv + h4) = __ldcg(reinterpret_cast<const float4 *>(a.w + i + h4));
+            *reinterpret_cast<float4 *>(m1 + h4) = __ldcg(reinterpret_cast<const float4 *>(a.m1 + i + h4));
+            *reinterpret_cast<float4 *>(m2 + h4) = __ldcg(reinterpret_cast<const float4 *>(a.m2 + i + h4));
+          }
+          bf16 b[8];
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            wv[e] = adam_one(ad, wv[e], v[e], m1[e], m2[e], true);
+            b[e] = __float2bfloat16_rn(wv[e]);
+          }
+#pragma unroll
+          for (int h4 = 0; h4 < 8; h4 += 4) {
+            *reinterpret_cast<float4 *>(a.w + i + h4) = *reinterpret_cast<const float4 *>(wv + h4);
+            *reinterpret_cast<float4 *>(a.m1 + i + h4) = *reinterpret_cast<const float4 *>(m1 + h4);
+            *reinterpret_cast<float4 *>(a.m2 + i + h4) = *reinterpret_cast<const float4 *>(m2 + h4);
+            if (keep_g) *reinterpret_cast<float4 *>(a.g + i + h4) = *reinterpret_cast<const float4 *>(v + h4);
+          }
+          *reinterpret_cast<uint4 *>(A.wb + (int64_t)row * A.in_k + c) = pack8(b);
+          if (A.wtb) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) A.wtb[(int64_t)(c + e) * A.ld_t + row] = b[e];
+          }
+        }
+      }
+      if (rank == kTrainCtas - 1) {  // output layer: D [input x output]
+        const AdamLayer &A = a.tab.l[L - 1];
+        float v[8];
+        tmem_ld8(trow + (uint32_t)(kGradCol + 32 * (L - 1) + half * 8), v);
+        bf16 b[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const int64_t j = (int64_t)(half * 8 + e) * A.in_k + row, i = A.w_off + j;
+          float m1 = __ldcg(a.m1 + i), m2 = __ldcg(a.m2 + i);
+          const float wn = adam_one(ad, __ldcg(a.w + i), v[e], m1, m2, true);
+          a.w[i] = wn;
+          a.m1[i] = m1;
+          a.m2[i] = m2;
+          if (keep_g) a.g[i] = v[e];
+          b[e] = __float2bfloat16_rn(wn);
+          A.wb[j] = b[e];
+        }
+        *reinterpret_cast<uint4 *>(A.wtb + (int64_t)row * A.ld_t + half * 8) = pack8(b);
+      }
+    }
+    tc_fence_before();
+    publish();
+    cluster_sync();
+  }
+  if (tid == 0) {
+    // copies issued before a wait gave up land before the CTA exits
+    for (; consumed < issued; ++consumed) mbar_wait(smem_u32(&bars[consumed % kTrainStages]), (consumed / kTrainStages) & 1u);
+    if (dead) atomicOr(a.err, 1u);
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
 // ---------------------------------------------------------------- host side
@@ -957,6 +1336,9 @@ struct mlp_handle_s {
   int nsm = 0;
   FusedArgs fa{};
   FusedMaps fm;
+  // training by k_train_cluster: its operand maps and a batch's partial losses
+  TrainMaps trm;
+  double *loss_part = nullptr;  // [cap / 128]
 };
 
 namespace {
@@ -1126,9 +1508,8 @@ int adam_step(mlp_handle *h) {
   h->t += 1;
   const double c1 = 1.0 - std::pow((double)h->p.beta1, (double)h->t);
   const double c2 = 1.0 - std::pow((double)h->p.beta2, (double)h->t);
-  k_adam<<<ceil_div(h->np_pad, 256), 256, 0, h->st>>>(h->w, h->g, h->m1, h->m2, h->np_pad, h->table, h->p.lr,
-                                                       h->p.beta1, h->p.beta2, h->p.eps, h->p.weight_decay,
-                                                       (float)c1, (float)c2);
+  const AdamStep k{h->p.lr, h->p.beta1, h->p.beta2, h->p.eps, h->p.weight_decay, (float)c1, (float)c2};
+  k_adam<<<ceil_div(h->np_pad, 256), 256, 0, h->st>>>(h->w, h->g, h->m1, h->m2, h->np_pad, h->table, k);
   OTF_LAUNCH_CHECK();
   return MD_OK;
 }
@@ -1186,7 +1567,7 @@ void destroy(mlp_handle *h) {
   mat_free(h->hi[1]);
   for (void *q : {(void *)h->w, (void *)h->g, (void *)h->m1, (void *)h->m2, (void *)h->xmean, (void *)h->xstd,
                   (void *)h->ymean, (void *)h->ystd, (void *)h->Y, (void *)h->T, (void *)h->loss, (void *)h->err,
-                  (void *)h->Yi})
+                  (void *)h->Yi, (void *)h->loss_part})
     if (q) cudaFree(q);
   if (h->err_host) cudaFreeHost(h->err_host);
   delete h;
@@ -1231,6 +1612,66 @@ int setup_fused(mlp_handle *h) {
   h->fused = h->p.width == kBM && need <= (size_t)optin;
   h->fused_smem = need;
   if (h->fused) OTF_CUDA(cudaFuncSetAttribute(k_mlp_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
+  return MD_OK;
+}
+
+// Operand maps of k_train_cluster that live as long as the handle (the
+// inputs' come with each mlp_train call).
+int setup_train(mlp_handle *h) {
+  TrainMaps &t = h->trm;
+  const int L = h->L;
+  auto slices = [](CUtensorMap *map, const Mat &M) { return make_map(map, M.p, (uint64_t)M.cols, (uint64_t)M.rows, 16); };
+  int rc = MD_OK;
+  for (int l = 0; l < L && !rc; ++l) {
+    rc = slices(&t.w[l], h->lay[l].wb);
+    if (!rc && l > 0) rc = slices(&t.wt[l], h->lay[l].wtb);
+    if (l == L - 1) break;
+    t.h[l] = h->H[l].map;
+    t.dz[l] = h->dZ[l].map;
+    t.dzt[l] = h->dZt[l].map;
+    if (!rc) rc = slices(&t.ht[l], h->Ht[l]);
+  }
+  t.ht_last = h->Ht[L - 2].map;
+  t.dy = h->dY.map;
+  t.dyt = h->dYt.map;
+  if (rc) return rc;
+  OTF_CUDA(cudaMalloc(&h->loss_part, sizeof(double) * (h->cap / kBM)));
+  OTF_CUDA(cudaFuncSetAttribute(k_train_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTrainSmem));
+  return MD_OK;
+}
+
+// The steps of one epoch: nb batches of the prepared inputs behind maps x, xt
+// and targets Ts; corr: their bias corrections (device).
+int train_epoch(mlp_handle *h, const Mat &Xs, const CUtensorMap &xt, const float *Ts, int64_t nb, const float2 *corr) {
+  TrainMaps tm = h->trm;
+  tm.x = Xs.map;
+  tm.xt = xt;
+  TrainArgs a{};
+  a.L = h->L;
+  a.n_out = h->p.n_out;
+  a.cap = h->cap;
+  a.nb = (int)nb;
+  a.tab = h->table;
+  a.adam = AdamStep{h->p.lr, h->p.beta1, h->p.beta2, h->p.eps, h->p.weight_decay, 0.f, 0.f};
+  a.corr = corr;
+  a.w = h->w, a.g = h->g, a.m1 = h->m1, a.m2 = h->m2;
+  for (int l = 0; l < h->L; ++l) a.in_k[l] = h->lay[l].in_k;
+  for (int l = 0; l < h->L - 1; ++l) {
+    a.H[l] = h->H[l].p;
+    a.Ht[l] = h->Ht[l].p;
+    a.dZ[l] = h->dZ[l].p;
+    a.dZt[l] = h->dZt[l].p;
+  }
+  a.dY = h->dY.p;
+  a.dYt = h->dYt.p;
+  a.Ts = Ts;
+  a.part = h->loss_part;
+  a.loss = h->loss;
+  a.acc_scale = 1.0 / (double)nb;  // the loss slot adds up to the epoch's mean
+  a.err = h->err;
+  a.wait_ns = h->wait_ns;
+  k_train_cluster<<<kTrainCtas, kTrainThreads, kTrainSmem, h->st>>>(tm, a);
+  OTF_LAUNCH_CHECK();
   return MD_OK;
 }
 
@@ -1322,6 +1763,7 @@ int create_impl(mlp_handle *h) {
   OTF_CUDA(cudaMallocHost(&h->err_host, sizeof(unsigned)));
   *h->err_host = 0u;
   OTF_CUDA(cudaDeviceSynchronize());
+  if (int rt = setup_train(h)) return rt;
   return setup_fused(h);
 }
 
@@ -1622,6 +2064,8 @@ int mlp_train(mlp_handle *h, const float *X, const float *T, int64_t rows, int32
   float *Tall = nullptr, *Ts = nullptr, *ox = nullptr, *ot = nullptr;
   int64_t *dperm = nullptr;
   double *dloss = nullptr;
+  float2 *dcorr = nullptr;  // [nb] bias corrections of an epoch's steps
+  CUtensorMap xt_map;
   const float *dX = nullptr, *dT = nullptr;
   std::vector<double> hist((size_t)epochs, 0.0);
   int rc = to_device(h, X, rows * h->p.n_in, mem, &ox, &dX);
@@ -1629,6 +2073,7 @@ int mlp_train(mlp_handle *h, const float *X, const float *T, int64_t rows, int32
   if (!rc) rc = mat_alloc(Xall, rows, h->k_in, kBM);
   if (!rc) rc = mat_alloc(Xs, nused, h->k_in, kBM);
   if (!rc) rc = mat_alloc(Xst, h->k_in, nused, (uint32_t)h->k_in);
+  if (!rc) rc = make_map(&xt_map, Xst.p, (uint64_t)Xst.cols, (uint64_t)Xst.rows, 16);
   auto cuda_ok = [&](cudaError_t e) {
     if (e != cudaSuccess && !rc) {
       set_error("mlp_train: %s", cudaGetErrorString(e));
@@ -1640,6 +2085,8 @@ int mlp_train(mlp_handle *h, const float *X, const float *T, int64_t rows, int32
   if (!rc) cuda_ok(cudaMalloc(&Ts, sizeof(float) * nused * h->p.n_out));
   if (!rc) cuda_ok(cudaMalloc(&dperm, sizeof(int64_t) * rows));
   if (!rc) cuda_ok(cudaMalloc(&dloss, sizeof(double) * std::max(epochs, 1)));
+  if (!rc) cuda_ok(cudaMalloc(&dcorr, sizeof(float2) * nb));
+  std::vector<float2> corr((size_t)nb);
   if (!rc) cuda_ok(cudaMemsetAsync(dloss, 0, sizeof(double) * std::max(epochs, 1), h->st));
   if (!rc) {
     k_prep_x<<<1024, 256, 0, h->st>>>(dX, rows, h->p.n_in, h->xmean, h->xstd, Xall.p, rows, h->k_in, nullptr, 0);
@@ -1670,11 +2117,13 @@ int mlp_train(mlp_handle *h, const float *X, const float *T, int64_t rows, int32
     if (!cuda_ok(cudaMemcpyAsync(dperm, perm.data(), sizeof(int64_t) * rows, cudaMemcpyHostToDevice, h->st))) break;
     k_gather<<<1024, 256, 0, h->st>>>(Xall.p, Tall, dperm, nused, h->k_in, h->p.n_out, Xs.p, Xst.p, Ts);
     if (!cuda_ok(cudaGetLastError())) break;
-    for (int64_t b = 0; b < nb && !rc; ++b) {
-      // the loss kernel adds loss / nb to the epoch's slot via h->loss[0]
-      rc = train_step(h, Xs, Xst, (int)(b * cap), Ts + b * cap * h->p.n_out, 1.0 / (double)nb);
-      if (!rc) rc = adam_step(h);
+    for (int64_t b = 0; b < nb; ++b) {
+      h->t += 1;
+      corr[(size_t)b] = make_float2((float)(1.0 - std::pow((double)h->p.beta1, (double)h->t)),
+                                    (float)(1.0 - std::pow((double)h->p.beta2, (double)h->t)));
     }
+    if (!cuda_ok(cudaMemcpyAsync(dcorr, corr.data(), sizeof(float2) * nb, cudaMemcpyHostToDevice, h->st))) break;
+    rc = train_epoch(h, Xs, xt_map, Ts, nb, dcorr);
     if (!rc) cuda_ok(cudaMemcpyAsync(dloss + e, h->loss, sizeof(double), cudaMemcpyDeviceToDevice, h->st));
     if (!rc) cuda_ok(cudaMemsetAsync(h->loss, 0, sizeof(double), h->st));
     if (!rc) cuda_ok(cudaStreamSynchronize(h->st));  // the host permutation buffer is reused next epoch
@@ -1687,7 +2136,7 @@ int mlp_train(mlp_handle *h, const float *X, const float *T, int64_t rows, int32
   mat_free(Xall);
   mat_free(Xs);
   mat_free(Xst);
-  for (void *q : {(void *)Tall, (void *)Ts, (void *)ox, (void *)ot, (void *)dperm, (void *)dloss})
+  for (void *q : {(void *)Tall, (void *)Ts, (void *)ox, (void *)ot, (void *)dperm, (void *)dloss, (void *)dcorr})
     if (q) cudaFree(q);
   return rc;
 }

@@ -231,3 +231,33 @@ def test_pipeline_wait_timeout_is_an_error_status(pkg, omlp):
     ye, _ = omlp.forward(params, X.astype(np.float64), True)
     assert loss == pytest.approx(omlp.loss(ye, T.astype(np.float64)), rel=1e-5)
     net.close()
+
+
+@pytest.mark.parametrize("n_in,depth,batch,batches", [(132, 3, 128, 3), (20, 1, 128, 2), (240, 2, 256, 2), (64, 6, 384, 2),
+                                                      (132, 3, 1152, 1)])
+def test_training_steps_equal_layered_steps(pkg, n_in, depth, batch, batches):
+    """mlp_train runs an epoch's steps in one launch; the same batches through
+    mlp_loss_grad and mlp_adam_step go layer by layer.  Both round at the same
+    points and add each element's products in the same order, so the weights
+    differ only by how an FP32 expression is contracted: a few units of the
+    largest weight's rounding (2^-24) per step, times the at most 2 lr that one
+    Adam step can move where a gradient is itself rounding noise."""
+    rows, lr = batch * batches, 1e-3
+    X = synth.normal(71, rows * n_in).reshape(rows, n_in).astype(np.float32)
+    T = synth.normal(72, rows * 2).reshape(rows, 2).astype(np.float32)
+    start = f32(synth.mlp_init(73, (n_in,) + (128,) * depth + (2,), bias_scale=0.1))
+    order = synth.permutations(74, 1, rows)
+    kw = dict(depth=depth, batch=batch, lr=lr, weight_decay=1e-3)
+    a, b = pkg.MLP(n_in, 2, **kw), pkg.MLP(n_in, 2, **kw)
+    a.set_params(start)
+    b.set_params(start)
+    hist = a.train(X, T, 1, order=order)
+    losses = []
+    for k in range(batches):
+        at = order[0, k * batch:(k + 1) * batch]
+        losses.append(b.loss_grad(X[at], T[at])[0])
+        b.adam_step()
+    assert hist[0] == pytest.approx(np.mean(losses), rel=1e-6)
+    d = np.abs(a.get_flat() - b.get_flat())
+    assert np.linalg.norm(d) <= 1e-5 * np.linalg.norm(b.get_flat())
+    assert d.max() <= 2.01 * lr * batches
