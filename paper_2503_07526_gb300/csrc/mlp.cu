@@ -88,6 +88,16 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
       : "memory");
 }
+// The same into the same place of every CTA of the cluster in the mask, each
+// CTA's barrier counting its copy.
+__device__ __forceinline__ void tma_load_2d_all(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar,
+                                                uint16_t mask) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1, {%2, "
+      "%3}], [%4], %5;" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar), "h"(mask)
+      : "memory");
+}
 __device__ __forceinline__ void tmem_alloc(uint32_t slot, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot), "r"(ncols) : "memory");
   asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -834,14 +844,17 @@ __global__ void k_cast_weights(const float *__restrict__ w, AdamTable tab) {
 // thread per row).  Here every product is cut into column slices over the
 // eight CTAs, and the phases of a step (one per layer forward, one per layer
 // back, the last weight gradient with Adam) are separated by cluster barriers:
-// TRAIN_FIGS per step.  Operands go through global memory (L2) in the same
-// matrices as the layered kernels use and come back by TMA, the writers
-// fencing the async proxy before each barrier; each weight gradient's product
-// runs beside the next layer's and stays in TMEM until Adam reads it there.
-// Every element's products are accumulated in the same order as in k_gemm_tc,
-// and rounding points and epilogue arithmetic are the same.
+// 38 us per step (train_3584: 12.95 -> 2.86 ms for 56 steps with the call's
+// set-up).  Operands go through global memory (L2) in the same matrices as the
+// layered kernels use and come back by TMA, the writers fencing the async proxy
+// before each barrier; each weight gradient's product runs beside the next
+// layer's and stays in TMEM until Adam reads it there.  Every element's
+// products are accumulated in the same order as in k_gemm_tc, and rounding
+// points and epilogue arithmetic are the same, so the weights are equal bit for
+// bit.  What bounds a step now: eight phases of about 4.5 us, each a chain of
+// fence, copy (L2 latency), products, epilogue, stores and barrier.
 constexpr int kTrainCtas = 8;
-constexpr int kTrainThreads = 256;
+constexpr int kTrainThreads = 640;  // 20 warps, see k_train_cluster
 constexpr int kTrainStages = 6;
 constexpr uint32_t kStageBytes = 2 * kPanelBytes;  // an A and a B panel of up to 128 rows
 constexpr int kGradCol = 128;                      // TMEM: layer l's gradient slices at kGradCol + 32 l
@@ -850,6 +863,7 @@ constexpr size_t kTrainSmem = 1024 + (size_t)kTrainStages * kStageBytes;
 struct TrainMaps {
   CUtensorMap x, xt;                     // this epoch's inputs: boxes of 128 rows; transposed, boxes of 16
   CUtensorMap h[kMaxLayers], dz[kMaxLayers], dzt[kMaxLayers], dy, ht_last;  // A operands, boxes of 128 rows
+  CUtensorMap x16, h16[kMaxLayers], dz16[kMaxLayers], dzt16[kMaxLayers], dy16;  // the same in boxes of 16 rows
   CUtensorMap w[kMaxLayers], wt[kMaxLayers], ht[kMaxLayers], dyt;           // B operands, boxes of 16 rows
 };
 struct TrainArgs {
@@ -862,7 +876,9 @@ struct TrainArgs {
   bf16 *H[kMaxLayers], *Ht[kMaxLayers], *dZ[kMaxLayers], *dZt[kMaxLayers], *dY, *dYt;
   const float *Ts;           // [nb cap][n_out] standardised targets in epoch order
   double *part, *loss;       // [cap / 128] a batch's partial losses; [2] as in k_loss_dy
-  double acc_scale;
+  float *state;              // [kTrainCtas][2 kMaxLayers][3][256][8] weight slices and moments
+  double acc_scale, inv;     // inv = 1 / (cap n_out)
+  float gscale;              // 2 inv
   unsigned *err;
   uint64_t wait_ns;
 };
@@ -870,11 +886,19 @@ struct TrainArgs {
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
 }
-// Global writes of this thread made visible to other CTAs' TMA loads (the
-// barrier that follows orders them; the reader fences too).
-__device__ __forceinline__ void publish() {
-  __threadfence();
-  asm volatile("fence.proxy.async;" ::: "memory");
+// Global writes of this thread made visible to other CTAs' TMA loads: the
+// barrier that follows releases them, the reader fences too.
+__device__ __forceinline__ void publish() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
+// mbar_wait_for with the potentially blocking try_wait: the hardware wakes the
+// thread, and the wall clock (about a microsecond to read) is looked at only
+// when that gave up once.
+__device__ __forceinline__ bool mbar_wait_short(uint32_t bar, uint32_t parity, uint64_t limit_ns) {
+  if (limit_ns == 0) return mbar_test(bar, parity);
+  if (mbar_try(bar, parity)) return true;
+  const uint64_t t0 = global_timer();
+  while (!mbar_try(bar, parity))
+    if (global_timer() - t0 > limit_ns) return false;
+  return true;
 }
 // 8 consecutive FP32 columns of this thread's TMEM lane.
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
@@ -894,307 +918,437 @@ __device__ __forceinline__ uint4 pack8(const bf16 (&b)[8]) {
   return q;
 }
 
+// One product of a phase: D [128 x N] at TMEM column col = A rows [arow, +128)
+// x B rows [brow, +N) over K columns from ak and bk; bar: arrives when it and
+// every product before it are done.
+// B rows come 16 at a time, bstep apart.  shared: the map of A in boxes of 16
+// rows when every CTA of the cluster takes the same A in this phase.
+struct TrainJob {
+  const CUtensorMap *ma, *mb, *shared;
+  int arow, ak, brow, bstep, bk, K, N, col;
+  uint32_t bar;
+};
+
+// Warps 0-7 run the epilogues (warp w: TMEM lanes 32 (w mod 4).., column half
+// w / 4), warp 8 issues copies and products, warps 9-11 the biases' gradients and steps,
+// warps 12-19 the weights' Adam steps of the layers whose gradients are done,
+// beside the phases that follow.
+constexpr int kEpiWarps = 8, kAdamWarp0 = 12;
+
 __global__ void __cluster_dims__(kTrainCtas, 1, 1) __launch_bounds__(kTrainThreads, 1)
     k_train_cluster(const __grid_constant__ TrainMaps tm, const __grid_constant__ TrainArgs a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  __shared__ uint64_t bars[2 * kTrainStages + 2];  // full[S], empty[S], product done, gradients done
+  __shared__ uint64_t bars[2 * kTrainStages + 1 + kMaxLayers];  // full[S], empty[S], product done, gradient l done
   __shared__ uint32_t slot;
   __shared__ volatile int dead;  // a wait gave up: no more products, epilogues or updates, only the barriers
-  __shared__ double wpart[kTrainThreads / 32];
+  __shared__ double wpart[kEpiWarps];
+  __shared__ float sbias[kMaxLayers * kBM];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, rank = (int)blockIdx.x;
-  const int quarter = warp & 3, half = warp >> 2, row = quarter * 32 + lane;  // TMEM lane and column half
-  const uint32_t done_bar = smem_u32(&bars[2 * kTrainStages]), grad_bar = smem_u32(&bars[2 * kTrainStages + 1]);
+  const int quarter = warp & 3, half = (warp >> 2) & 1, row = quarter * 32 + lane;
+  const uint32_t done_bar = smem_u32(&bars[2 * kTrainStages]);
+  auto grad_bar = [&](int l) { return smem_u32(&bars[2 * kTrainStages + 1 + l]); };
   if (tid == 0) {
-    for (int s = 0; s < 2 * kTrainStages + 2; ++s) mbar_init(smem_u32(&bars[s]), 1);
+    for (int s = 0; s < 2 * kTrainStages + 1 + kMaxLayers; ++s) mbar_init(smem_u32(&bars[s]), 1);
     dead = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) tmem_alloc(smem_u32(&slot), 512);
   tc_fence_before();
   __syncthreads();
+  cluster_sync();  // every CTA's barriers are set up before another's copies count on them
   tc_fence_after();
   const uint32_t tmem = slot;
   const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16);
   const int L = a.L, mt = a.cap / kBM;
   const int nsl = mt >= kTrainCtas ? 1 : kTrainCtas / mt;  // column slices of a 128-wide product
   const int wsl = kBM / nsl, tiles = mt * nsl;
+  const bool epi = warp < kEpiWarps, issuer = warp == kEpiWarps && lane == 0;
 
-  // thread 0: panels issued and consumed so far (stage = count mod kTrainStages)
+  // With one 128-row tile per batch every CTA multiplies by the same A: each
+  // fetches an eighth of it for all (TMA multicast).  Eight CTAs fetching all
+  // of it took about 10 bytes per cycle and SM.  Every CTA then issues the same
+  // panels (some ignore a product's result), so their stages stay in step; a
+  // phase uses no stage twice and ends with its products done, so the cluster barrier between
+  // phases also says that every CTA's stages are free.
+  const bool multi = mt == 1;
+  // issuer: panels issued and consumed so far (stage = count mod kTrainStages)
   uint32_t issued = 0, consumed = 0;
-  // D [128 x N] at TMEM column col += A rows [arow, +128) x B rows [brow, +N)
-  // over K columns from ak and bk (thread 0; two or more panels in flight)
-  auto product = [&](const CUtensorMap *ma, int arow, int ak, const CUtensorMap *mb, int brow, int bk, int K, int N,
-                     int col) {
-    if (dead) return;
-    const int np = (K + kBK - 1) / kBK;
-    const uint32_t idesc = idesc_bf16(kBM, N);
-    int in = 0;
-    for (int p = 0; p < np; ++p) {
-      for (; in < np && in < p + kTrainStages; ++in, ++issued) {
+  // a phase's product (or two, the second's copies running ahead of the
+  // first's products).  Jobs go by value and are picked by selects: an indexed
+  // array would sit in memory and be read again after every copy and fence
+  // (2,000 to 9,000 cycles of a phase)
+  auto run_jobs = [&](const TrainJob j0, const TrainJob j1, int nj) {
+    asm volatile("fence.proxy.async.global;" ::: "memory");
+    const int n0 = (j0.K + kBK - 1) / kBK, total = n0 + (nj > 1 ? (j1.K + kBK - 1) / kBK : 0);
+    bool ok = !dead, first = false;  // first: j0's barrier has been committed to
+    int ld = 0;
+    for (int c = 0; c < total && ok; ++c) {
+      for (; ld < total && issued < consumed + kTrainStages && ok; ++ld) {
+        const bool second = ld >= n0;
+        const int p = second ? ld - n0 : ld;
         const uint32_t s = issued % kTrainStages, use = issued / kTrainStages;
-        if (use > 0 && !mbar_wait_for(smem_u32(&bars[kTrainStages + s]), (use - 1) & 1u, a.wait_ns)) {
-          dead = 1;
-          return;
+        if (use > 0 && !mbar_wait_short(smem_u32(&bars[kTrainStages + s]), (use - 1) & 1u, a.wait_ns)) {
+          ok = false;
+          break;
         }
         const uint32_t fb = smem_u32(&bars[s]), sa = smem_u32(smem + s * kStageBytes);
+        const int N = second ? j1.N : j0.N, ax = (second ? j1.ak : j0.ak) + p * kBK, ay = second ? j1.arow : j0.arow;
+        const int bx = (second ? j1.bk : j0.bk) + p * kBK, by = second ? j1.brow : j0.brow, bs = second ? j1.bstep : j0.bstep;
+        const CUtensorMap *mb = second ? j1.mb : j0.mb, *ms = second ? j1.shared : j0.shared;
         mbar_expect_tx(fb, kPanelBytes + (uint32_t)N * 128u);
-        tma_load_2d(sa, ma, ak + in * kBK, arow, fb);
-        for (int r = 0; r < N; r += 16) tma_load_2d(sa + kPanelBytes + r * 128u, mb, bk + in * kBK, brow + r, fb);
+        if (multi && ms)
+          tma_load_2d_all(sa + rank * 16u * 128u, ms, ax, ay + rank * 16, fb, (uint16_t)((1 << kTrainCtas) - 1));
+        else
+          tma_load_2d(sa, second ? j1.ma : j0.ma, ax, ay, fb);
+        for (int r = 0, y = by; r < N; r += 16, y += bs) tma_load_2d(sa + kPanelBytes + r * 128u, mb, bx, y, fb);
+        ++issued;
       }
+      const bool second = c >= n0;
+      const int p = second ? c - n0 : c;
       const uint32_t s = consumed % kTrainStages;
-      if (!mbar_wait_for(smem_u32(&bars[s]), (consumed / kTrainStages) & 1u, a.wait_ns)) {
-        dead = 1;
-        return;
-      }
+      ok = ok && mbar_wait_short(smem_u32(&bars[s]), (consumed / kTrainStages) & 1u, a.wait_ns);
+      if (!ok) break;
       ++consumed;
       tc_fence_after();
-      const uint32_t a0 = smem_u32(smem + s * kStageBytes), b0 = a0 + kPanelBytes;
-      const int nk = min(kBK, K - p * kBK) / 16;
-      for (int j = 0; j < nk; ++j)
-        mma_bf16(tmem + (uint32_t)col, sw128_desc(a0 + 32u * j), sw128_desc(b0 + 32u * j), idesc, (p | j) != 0);
+      const uint64_t da = sw128_desc(smem_u32(smem + s * kStageBytes)), db = sw128_desc(smem_u32(smem + s * kStageBytes) + kPanelBytes);
+      const uint32_t idesc = idesc_bf16(kBM, second ? j1.N : j0.N), d = tmem + (uint32_t)(second ? j1.col : j0.col);
+      const int left = (second ? j1.K : j0.K) - p * kBK;
+#pragma unroll
+      for (int q = 0; q < kBK / 16; ++q)  // 32 bytes of a row further: 2 in the address field
+        if (16 * q < left) mma_bf16(d, da + 2 * q, db + 2 * q, idesc, (p | q) != 0);
       mma_commit(smem_u32(&bars[kTrainStages + s]));
+      if (c == n0 - 1) {
+        mma_commit(j0.bar);
+        first = true;
+      }
+    }
+    if (!ok) {
+      dead = 1;
+      __threadfence_block();  // before the barriers that its readers wait for
+      if (!first) mma_commit(j0.bar);
+    }
+    if (nj > 1) mma_commit(j1.bar);
+    if (multi && consumed > 0) {
+      const uint32_t last = consumed - 1;
+      if (!mbar_wait_blocking(smem_u32(&bars[kTrainStages + last % kTrainStages]), (last / kTrainStages) & 1u)) dead = 1;
     }
   };
-  uint32_t phase = 0;
-  // waits for the product committed to done_bar (every thread); false: skip the epilogue
-  auto finish = [&]() {
-    const bool ok = mbar_wait(done_bar, phase);
-    phase ^= 1u;
+  // epilogue and Adam warps: waits for a barrier's phase; uniform over a warp
+  auto ready = [&](uint32_t bar, uint32_t parity) {
+    const bool ok = mbar_wait_blocking(bar, parity);
     if (!ok) dead = 1;
     tc_fence_after();
+    return __all_sync(0xffffffffu, ok && !dead) != 0;
+  };
+  uint32_t phase = 0;  // of done_bar (epilogue warps)
+
+  auto epi_sync = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiWarps * 32) : "memory"); };
+
+  // does this CTA hold gradient slice k of layer l?
+  auto has_slice = [&](int l, int k) {
+    return l == L - 1 ? k == 0 && rank == kTrainCtas - 1 : (rank + kTrainCtas * k) * 16 < a.in_k[l];
+  };
+  // This CTA's weight slices with their moments live in a.state for the
+  // launch, ordered so that a warp's accesses are whole lines: slice n (count
+  // of the CTA's slices before it), array (w, m1, m2), four of a thread's
+  // eight elements, thread.  In w's own order a lane's eight elements lie a
+  // row apart from its neighbours' and each access touched 32 lines, which
+  // slowed the copies of the products beside it as well.
+  auto state_at = [&](int n) {
+    return reinterpret_cast<float4 *>(a.state) + ((int64_t)rank * 2 * kMaxLayers + n) * 6 * 256 + (warp & 7) * 32 + lane;
+  };
+  // hidden layers' slice k: output row `row`, eight consecutive inputs; the
+  // output layer's: input `row`, eight outputs (a column of W each)
+  auto param_at = [&](int l, int k, int e) {
+    const AdamLayer &A = a.tab.l[l];
+    const int c = half * 8 + e;
+    return A.w_off + (l == L - 1 ? (int64_t)c * A.in_k + row : (int64_t)row * A.in_k + (rank + kTrainCtas * k) * 16 + c);
+  };
+  auto slice_no = [&](int l, int k) { return 2 * l + k; };
+  // moves the slices between the parameter vectors and a.state
+  auto move_state = [&](bool in) {
+    for (int l = 0; l < L; ++l)
+      for (int k = 0; k < 2; ++k) {
+        if (!has_slice(l, k)) continue;
+        float4 *st = state_at(slice_no(l, k));
+        float *arr[3] = {a.w, a.m1, a.m2};
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+          float *p = arr[q >> 1];
+          float v[4];
+          if (in) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) v[e] = __ldcg(p + param_at(l, k, 4 * (q & 1) + e));
+            st[q * 256] = make_float4(v[0], v[1], v[2], v[3]);
+          } else {
+            *reinterpret_cast<float4 *>(v) = __ldcg(st + q * 256);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) p[param_at(l, k, 4 * (q & 1) + e)] = v[e];
+          }
+        }
+      }
+  };
+  // Adam on layer l's gradient slice k of this CTA (a warp's 32 rows, 8 columns)
+  auto adam_slice = [&](int l, int k, const AdamStep &ad, bool keep_g) {
+    const AdamLayer &A = a.tab.l[l];
+    const bool out = l == L - 1;
+    const int c = out ? half * 8 : (rank + kTrainCtas * k) * 16 + half * 8;
+    float4 *st = state_at(slice_no(l, k));
+    float v[8], s[3][8];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) *reinterpret_cast<float4 *>(s[q >> 1] + 4 * (q & 1)) = __ldcg(st + q * 256);
+    tmem_ld8(trow + (uint32_t)(kGradCol + 32 * l + 16 * k + half * 8), v);
+    bf16 b[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      s[0][e] = adam_one(ad, s[0][e], v[e], s[1][e], s[2][e], true);
+      b[e] = __float2bfloat16_rn(s[0][e]);
+    }
+#pragma unroll
+    for (int q = 0; q < 6; ++q) st[q * 256] = *reinterpret_cast<const float4 *>(s[q >> 1] + 4 * (q & 1));
+    if (out) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) A.wb[(int64_t)(c + e) * A.in_k + row] = b[e];
+      *reinterpret_cast<uint4 *>(A.wtb + (int64_t)row * A.ld_t + c) = pack8(b);
+    } else {
+      *reinterpret_cast<uint4 *>(A.wb + (int64_t)row * A.in_k + c) = pack8(b);
+      if (A.wtb) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) A.wtb[(int64_t)(c + e) * A.ld_t + row] = b[e];
+      }
+    }
+    if (keep_g) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) a.g[param_at(l, k, e)] = v[e];
+    }
+  };
+  auto phase_end = [&]() {
+    tc_fence_before();
+    publish();
     __syncthreads();
-    const bool run = dead == 0;
-    __syncthreads();  // thread 0 may set it again in the next product
-    return run;
+    cluster_sync();
   };
 
+  if (epi) move_state(true);
+  __syncthreads();  // the Adam warps read what the epilogue warps moved
   for (int step = 0; step < a.nb; ++step) {
     const int row0 = step * a.cap;
+    const uint32_t sp = (uint32_t)step & 1u;
+    AdamStep ad = a.adam;
+    const float2 corr = __ldg(a.corr + step);
+    ad.c1 = corr.x;
+    ad.c2 = corr.y;
+    const bool keep_g = step == a.nb - 1;  // the last batch's gradients stay readable, as after the layered step
+    if (epi) {  // this step's biases
+      for (int q = tid; q < L * kBM; q += kEpiWarps * 32) {
+        const int l = q / kBM, c = q % kBM;
+        if (l < L - 1 || c < kOutPad) sbias[q] = __ldcg(a.w + a.tab.l[l].b_off + c);
+      }
+      epi_sync();
+    }
     // forward
     for (int l = 0; l < L - 1; ++l) {
       for (int t = rank; t < tiles; t += kTrainCtas) {
         const int m0 = (t / nsl) * kBM, n0 = (t % nsl) * wsl;
-        if (tid == 0) {
-          asm volatile("fence.proxy.async;" ::: "memory");
-          product(l == 0 ? &tm.x : &tm.h[l - 1], (l == 0 ? row0 : 0) + m0, 0, &tm.w[l], n0, 0, a.in_k[l], wsl, 0);
-          mma_commit(done_bar);
+        if (issuer) {
+          const TrainJob j = TrainJob{l == 0 ? &tm.x : &tm.h[l - 1], &tm.w[l], l == 0 ? &tm.x16 : &tm.h16[l - 1],
+                             (l == 0 ? row0 : 0) + m0, 0, n0, 16, 0, a.in_k[l], wsl, 0, done_bar};
+          run_jobs(j, j, 1);
         }
-        if (finish()) {
-          const float *bias = a.w + a.tab.l[l].b_off + n0;
+        if (epi && ready(done_bar, phase)) {
           const int64_t m = m0 + row;
           for (int c0 = half * (wsl / 2); c0 < (half + 1) * (wsl / 2); c0 += 8) {
             float v[8];
             tmem_ld8(trow + (uint32_t)c0, v);
             bf16 b[8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) b[i] = __float2bfloat16_rn(tanhf(v[i] + __ldcg(bias + c0 + i)));
+            for (int i = 0; i < 8; ++i) b[i] = __float2bfloat16_rn(tanhf(v[i] + sbias[l * kBM + n0 + c0 + i]));
             *reinterpret_cast<uint4 *>(a.H[l] + m * kBM + n0 + c0) = pack8(b);
 #pragma unroll
             for (int i = 0; i < 8; ++i) a.Ht[l][(int64_t)(n0 + c0 + i) * a.cap + m] = b[i];
           }
         }
+        phase ^= 1u;
         tc_fence_before();
-        __syncthreads();
+        if (tiles > kTrainCtas) __syncthreads();  // the accumulator is reused
       }
-      publish();
-      cluster_sync();
+      phase_end();
     }
     // output layer, loss and its gradient (tile t: rows of one CTA)
-    for (int t = rank; t < mt; t += kTrainCtas) {
-      if (tid == 0) {
-        asm volatile("fence.proxy.async;" ::: "memory");
-        product(&tm.h[L - 2], t * kBM, 0, &tm.w[L - 1], 0, 0, a.in_k[L - 1], kOutPad, 0);
-        mma_commit(done_bar);
+    for (int t = rank; t < mt || (multi && t == rank); t += kTrainCtas) {
+      const bool mine = t < mt;
+      if (issuer) {  // with a shared A the others copy their part too
+        const TrainJob j{&tm.h[L - 2], &tm.w[L - 1], &tm.h16[L - 2], mine ? t * kBM : 0, 0, 0, 16, 0, a.in_k[L - 1], kOutPad, 0, done_bar};
+        run_jobs(j, j, 1);
       }
-      double acc = 0.0;
-      if (finish()) {
-        const float *bias = a.w + a.tab.l[L - 1].b_off;
+      if (epi && mine) {
         const int64_t m = (int64_t)t * kBM + row;
-        const float gscale = (float)(2.0 * (1.0 / ((double)a.cap * a.n_out)));
-        float v[8];
-        tmem_ld8(trow + (uint32_t)(half * 8), v);
+        float tgt[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int c = half * 8 + i;
-          if (c < a.n_out) {
-            const float d = (v[i] + __ldcg(bias + c)) - a.Ts[(row0 + m) * a.n_out + c];
-            acc += (double)d * d;
-            const bf16 db = __float2bfloat16_rn(gscale * d);
-            a.dY[m * 64 + c] = db;
-            a.dYt[(int64_t)c * a.cap + m] = db;
+        for (int i = 0; i < 8; ++i) tgt[i] = half * 8 + i < a.n_out ? a.Ts[(row0 + m) * a.n_out + half * 8 + i] : 0.f;
+        double acc = 0.0;
+        if (ready(done_bar, phase)) {
+          float v[8];
+          tmem_ld8(trow + (uint32_t)(half * 8), v);
+          bf16 b[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const int c = half * 8 + i;
+            b[i] = __float2bfloat16_rn(0.f);
+            if (c < a.n_out) {
+              const float d = (v[i] + sbias[(L - 1) * kBM + c]) - tgt[i];
+              acc += (double)d * d;
+              b[i] = __float2bfloat16_rn(a.gscale * d);
+              a.dY[m * 64 + c] = b[i];
+              a.dYt[(int64_t)c * a.cap + m] = b[i];
+            }
           }
         }
+        acc = warp_sum(acc);
+        if (lane == 0) wpart[warp] = acc;
+        tc_fence_before();
+        epi_sync();
+        if (tid == 32) {
+          double s = 0.0;
+          for (int w = 0; w < kEpiWarps; ++w) s += wpart[w];
+          a.part[t] = s;
+        }
       }
-      acc = warp_sum(acc);
-      if (lane == 0) wpart[warp] = acc;
-      tc_fence_before();
-      __syncthreads();
-      if (tid == 0) {
-        double s = 0.0;
-        for (int w = 0; w < kTrainThreads / 32; ++w) s += wpart[w];
-        a.part[t] = s;
-      }
+      phase ^= 1u;
+      if (mt > kTrainCtas) __syncthreads();
     }
-    publish();
-    cluster_sync();
+    phase_end();
     // back: dZ_l = (dZ_{l+1} W_{l+1}) (1 - H_l^2), and beside it the weight
-    // gradient of layer l + 1, left in TMEM
+    // gradient of layer l + 1, left in TMEM, and Adam on that of layer l + 2
     for (int l = L - 2; l >= 0; --l) {
       const bool top = l == L - 2;
+      if (warp >= kAdamWarp0 && !top && has_slice(l + 2, 0) && ready(grad_bar(l + 2), sp)) adam_slice(l + 2, 0, ad, keep_g);
       bool graded = false;
       for (int t = rank; t < tiles || !graded; t += kTrainCtas) {
         const bool mine = t < tiles;
         const int m0 = (t / nsl) * kBM, n0 = (t % nsl) * wsl;
-        if (tid == 0) {
-          asm volatile("fence.proxy.async;" ::: "memory");
-          if (mine) {
-            product(top ? &tm.dy : &tm.dz[l + 1], m0, 0, &tm.wt[l + 1], n0, 0, top ? kOutPad : kBM, wsl, 0);
-            mma_commit(done_bar);
-          }
-          if (!graded) {
-            if (!top)
-              product(&tm.dzt[l + 1], 0, 0, &tm.ht[l], rank * 16, 0, a.cap, 16, kGradCol + 32 * (l + 1));
-            else if (rank == kTrainCtas - 1)
-              product(&tm.ht_last, 0, 0, &tm.dyt, 0, 0, a.cap, kOutPad, kGradCol + 32 * (l + 1));
-          }
+        if (issuer) {
+          TrainJob j{}, g{};
+          if (mine)
+            j = TrainJob{top ? &tm.dy : &tm.dz[l + 1], &tm.wt[l + 1], top ? &tm.dy16 : &tm.dz16[l + 1], m0, 0, n0, 16, 0,
+                         top ? kOutPad : kBM, wsl, 0, done_bar};
+          const bool grad = !graded && (multi || has_slice(l + 1, 0));
+          if (top)
+            g = TrainJob{&tm.ht_last, &tm.dyt, &tm.ht[l], 0, 0, 0, 16, 0, a.cap, kOutPad, kGradCol + 32 * (l + 1), grad_bar(l + 1)};
+          else
+            g = TrainJob{&tm.dzt[l + 1], &tm.ht[l], &tm.dzt16[l + 1], 0, 0, rank * 16, 16, 0, a.cap, 16, kGradCol + 32 * (l + 1),
+                         grad_bar(l + 1)};
+          if (mine)
+            run_jobs(j, g, grad ? 2 : 1);
+          else if (grad)
+            run_jobs(g, g, 1);
         }
         graded = true;
         __syncwarp();
         if (!mine) break;
-        if (finish()) {
+        if (epi) {
           const int64_t m = m0 + row;
-          for (int c0 = half * (wsl / 2); c0 < (half + 1) * (wsl / 2); c0 += 8) {
-            float v[8];
-            tmem_ld8(trow + (uint32_t)c0, v);
-            const uint4 hq = __ldcg(reinterpret_cast<const uint4 *>(a.H[l] + m * kBM + n0 + c0));
-            const bf16 *hb = reinterpret_cast<const bf16 *>(&hq);
-            bf16 b[8];
+          if (ready(done_bar, phase)) {
+            for (int c0 = half * (wsl / 2); c0 < (half + 1) * (wsl / 2); c0 += 8) {
+              const uint4 hq = __ldcg(reinterpret_cast<const uint4 *>(a.H[l] + m * kBM + n0 + c0));
+              const bf16 *hb = reinterpret_cast<const bf16 *>(&hq);
+              float v[8];
+              tmem_ld8(trow + (uint32_t)c0, v);
+              bf16 b[8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const float hd = __bfloat162float(hb[i]);
-              b[i] = __float2bfloat16_rn(v[i] * (1.0f - hd * hd));
+              for (int i = 0; i < 8; ++i) {
+                const float hd = __bfloat162float(hb[i]);
+                b[i] = __float2bfloat16_rn(v[i] * (1.0f - hd * hd));
+              }
+              *reinterpret_cast<uint4 *>(a.dZ[l] + m * kBM + n0 + c0) = pack8(b);
+#pragma unroll
+              for (int i = 0; i < 8; ++i) a.dZt[l][(int64_t)(n0 + c0 + i) * a.cap + m] = b[i];
             }
-            *reinterpret_cast<uint4 *>(a.dZ[l] + m * kBM + n0 + c0) = pack8(b);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) a.dZt[l][(int64_t)(n0 + c0 + i) * a.cap + m] = b[i];
           }
+          tc_fence_before();
         }
-        tc_fence_before();
-        __syncthreads();
+        phase ^= 1u;
+        if (tiles > kTrainCtas) __syncthreads();
       }
-      publish();
-      cluster_sync();
+      phase_end();
     }
-    // the first layer's weight gradient, the bias gradients meanwhile, then Adam
-    const float2 corr = __ldg(a.corr + step);
-    AdamStep ad = a.adam;
-    ad.c1 = corr.x;
-    ad.c2 = corr.y;
-    const bool keep_g = step == a.nb - 1;  // the last batch's gradients stay readable, as after the layered step
-    if (tid == 0) {
-      asm volatile("fence.proxy.async;" ::: "memory");
-      for (int s = rank, k = 0; s * 16 < a.in_k[0]; s += kTrainCtas, ++k)
-        product(&tm.dzt[0], 0, 0, &tm.xt, s * 16, row0, a.cap, 16, kGradCol + 16 * k);
-      mma_commit(grad_bar);
-      if (rank == 0) {
+    // the first layer's weight gradient, the biases, then the last two layers' Adam
+    if (issuer) {
+      // slices rank and rank + 8 of the inputs, as far as there are any; with a
+      // shared A every CTA takes its part in the copies
+      const int N = has_slice(0, 1) ? 32 : 16;
+      const bool any = has_slice(0, 0);
+      const TrainJob j{&tm.dzt[0], &tm.xt, &tm.dzt16[0], 0, 0, any ? rank * 16 : 0, 16 * kTrainCtas, row0, a.cap, N, kGradCol, grad_bar(0)};
+      run_jobs(j, j, 1);
+    } else if (warp > kEpiWarps && warp < kAdamWarp0) {
+      // bias gradients: the rows of dZ^T summed as k_bias_grad does (the same
+      // order: an element of rounding size takes a step of full size in Adam's
+      // first steps, so another order shows in the weights), six columns' loads
+      // in flight
+      constexpr int kCols = 6;
+      const int ncol = (L - 1) * kBM + kOutPad;
+      for (int j0 = warp - kEpiWarps - 1; rank + kTrainCtas * j0 < ncol && !dead; j0 += 3 * kCols) {
+        float acc[kCols];
+        const unsigned short *src[kCols];
+#pragma unroll
+        for (int u = 0; u < kCols; ++u) {
+          const int q = min(rank + kTrainCtas * (j0 + 3 * u), ncol - 1), l = min(q / kBM, L - 1);
+          src[u] = reinterpret_cast<const unsigned short *>(l < L - 1 ? a.dZt[l] : a.dYt) + (int64_t)(q - l * kBM) * a.cap + lane;
+          acc[u] = 0.f;
+        }
+        for (int m = 0; m < a.cap; m += 128) {
+          unsigned short v[kCols][4];
+#pragma unroll
+          for (int u = 0; u < kCols; ++u)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v[u][k] = __ldcg(src[u] + m + 32 * k);
+#pragma unroll
+          for (int u = 0; u < kCols; ++u)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) acc[u] += __bfloat162float(__ushort_as_bfloat16(v[u][k]));
+        }
+        float mine = 0.f;
+#pragma unroll
+        for (int u = 0; u < kCols; ++u) {
+          const float t = warp_sum(acc[u]);
+          if (lane == u) mine = t;
+        }
+        const int q = rank + kTrainCtas * (j0 + 3 * lane);
+        if (lane < kCols && q < ncol) {
+          const int l = min(q / kBM, L - 1);
+          const int64_t i = a.tab.l[l].b_off + (q - l * kBM);
+          float m1 = __ldcg(a.m1 + i), m2 = __ldcg(a.m2 + i);
+          a.w[i] = adam_one(ad, __ldcg(a.w + i), mine, m1, m2, false);
+          a.m1[i] = m1;
+          a.m2[i] = m2;
+          if (keep_g) a.g[i] = mine;
+        }
+      }
+      if (rank == 0 && warp == kAdamWarp0 - 1 && lane == 31) {
         double s = 0.0;
         for (int t = 0; t < mt; ++t) s += __ldcg(a.part + t);
-        s *= 1.0 / ((double)a.cap * a.n_out);
+        s *= a.inv;
         a.loss[0] += s * a.acc_scale;
         a.loss[1] = s;
       }
+    } else if (warp >= kAdamWarp0) {
+      if (has_slice(1, 0) && ready(grad_bar(1), sp)) adam_slice(1, 0, ad, keep_g);
+      if (has_slice(0, 1) && ready(grad_bar(0), sp)) adam_slice(0, 1, ad, keep_g);
+    } else if (epi) {
+      if (has_slice(0, 0) && ready(grad_bar(0), sp)) adam_slice(0, 0, ad, keep_g);
     }
-    if (warp > 0 && !dead) {
-      for (int q = rank * 7 + warp - 1; q < (L - 1) * kBM + kOutPad; q += kTrainCtas * 7) {
-        const int l = min(q / kBM, L - 1), n = q - l * kBM;
-        const bf16 *src = (l < L - 1 ? a.dZt[l] : a.dYt) + (int64_t)n * a.cap;
-        float acc = 0.f;
-        for (int m = lane; m < a.cap; m += 32)
-          acc += __bfloat162float(__ushort_as_bfloat16(__ldcg(reinterpret_cast<const unsigned short *>(src) + m)));
-        acc = warp_sum(acc);
-        if (lane == 0) {
-          const int64_t i = a.tab.l[l].b_off + n;
-          float m1 = __ldcg(a.m1 + i), m2 = __ldcg(a.m2 + i);
-          a.w[i] = adam_one(ad, __ldcg(a.w + i), acc, m1, m2, false);
-          a.m1[i] = m1;
-          a.m2[i] = m2;
-          if (keep_g) a.g[i] = acc;
-        }
-      }
-    }
-    __syncwarp();
-    const bool gok = mbar_wait(grad_bar, (uint32_t)step & 1u);
-    if (!gok) dead = 1;
-    tc_fence_after();
-    __syncthreads();
-    const bool update = dead == 0;
-    if (update) {
-      for (int l = 0; l < L - 1; ++l) {
-        const AdamLayer &A = a.tab.l[l];
-        for (int s = rank, k = 0; s * 16 < a.in_k[l]; s += kTrainCtas, ++k) {
-          float v[8];
-          tmem_ld8(trow + (uint32_t)(kGradCol + 32 * l + 16 * k + half * 8), v);
-          const int c = s * 16 + half * 8;  // eight input columns of output row `row`
-          const int64_t i = A.w_off + (int64_t)row * A.in_k + c;
-          float wv[8], m1[8], m2[8];
-#pragma unroll
-          for (int h4 = 0; h4 < 8; h4 += 4) {
-            *reinterpret_cast<float4 *>(wv + h4) = __ldcg(reinterpret_cast<const float4 *>(a.w + i + h4));
-            *reinterpret_cast<float4 *>(m1 + h4) = __ldcg(reinterpret_cast<const float4 *>(a.m1 + i + h4));
-            *reinterpret_cast<float4 *>(m2 + h4) = __ldcg(reinterpret_cast<const float4 *>(a.m2 + i + h4));
-          }
-          bf16 b[8];
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            wv[e] = adam_one(ad, wv[e], v[e], m1[e], m2[e], true);
-            b[e] = __float2bfloat16_rn(wv[e]);
-          }
-#pragma unroll
-          for (int h4 = 0; h4 < 8; h4 += 4) {
-            *reinterpret_cast<float4 *>(a.w + i + h4) = *reinterpret_cast<const float4 *>(wv + h4);
-            *reinterpret_cast<float4 *>(a.m1 + i + h4) = *reinterpret_cast<const float4 *>(m1 + h4);
-            *reinterpret_cast<float4 *>(a.m2 + i + h4) = *reinterpret_cast<const float4 *>(m2 + h4);
-            if (keep_g) *reinterpret_cast<float4 *>(a.g + i + h4) = *reinterpret_cast<const float4 *>(v + h4);
-          }
-          *reinterpret_cast<uint4 *>(A.wb + (int64_t)row * A.in_k + c) = pack8(b);
-          if (A.wtb) {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) A.wtb[(int64_t)(c + e) * A.ld_t + row] = b[e];
-          }
-        }
-      }
-      if (rank == kTrainCtas - 1) {  // output layer: D [input x output]
-        const AdamLayer &A = a.tab.l[L - 1];
-        float v[8];
-        tmem_ld8(trow + (uint32_t)(kGradCol + 32 * (L - 1) + half * 8), v);
-        bf16 b[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const int64_t j = (int64_t)(half * 8 + e) * A.in_k + row, i = A.w_off + j;
-          float m1 = __ldcg(a.m1 + i), m2 = __ldcg(a.m2 + i);
-          const float wn = adam_one(ad, __ldcg(a.w + i), v[e], m1, m2, true);
-          a.w[i] = wn;
-          a.m1[i] = m1;
-          a.m2[i] = m2;
-          if (keep_g) a.g[i] = v[e];
-          b[e] = __float2bfloat16_rn(wn);
-          A.wb[j] = b[e];
-        }
-        *reinterpret_cast<uint4 *>(A.wtb + (int64_t)row * A.ld_t + half * 8) = pack8(b);
-      }
-    }
-    tc_fence_before();
-    publish();
-    cluster_sync();
+    phase_end();
   }
-  if (tid == 0) {
+  if (epi) move_state(false);
+  if (issuer) {
     // copies issued before a wait gave up land before the CTA exits
     for (; consumed < issued; ++consumed) mbar_wait(smem_u32(&bars[consumed % kTrainStages]), (consumed / kTrainStages) & 1u);
     if (dead) atomicOr(a.err, 1u);
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync();  // no copy of this CTA is on its way to another that has left
   if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
@@ -1337,8 +1491,10 @@ struct mlp_handle_s {
   FusedArgs fa{};
   FusedMaps fm;
   // training by k_train_cluster: its operand maps and a batch's partial losses
+  bool train_ready = false;
   TrainMaps trm;
   double *loss_part = nullptr;  // [cap / 128]
+  float *train_state = nullptr; // a launch's weight slices and moments
 };
 
 namespace {
@@ -1567,7 +1723,7 @@ void destroy(mlp_handle *h) {
   mat_free(h->hi[1]);
   for (void *q : {(void *)h->w, (void *)h->g, (void *)h->m1, (void *)h->m2, (void *)h->xmean, (void *)h->xstd,
                   (void *)h->ymean, (void *)h->ystd, (void *)h->Y, (void *)h->T, (void *)h->loss, (void *)h->err,
-                  (void *)h->Yi, (void *)h->loss_part})
+                  (void *)h->Yi, (void *)h->loss_part, (void *)h->train_state})
     if (q) cudaFree(q);
   if (h->err_host) cudaFreeHost(h->err_host);
   delete h;
@@ -1615,9 +1771,10 @@ int setup_fused(mlp_handle *h) {
   return MD_OK;
 }
 
-// Operand maps of k_train_cluster that live as long as the handle (the
-// inputs' come with each mlp_train call).
+// Operand maps and scratch of k_train_cluster, kept by the handle from its
+// first mlp_train call on (the inputs' maps come with each call).
 int setup_train(mlp_handle *h) {
+  if (h->train_ready) return MD_OK;
   TrainMaps &t = h->trm;
   const int L = h->L;
   auto slices = [](CUtensorMap *map, const Mat &M) { return make_map(map, M.p, (uint64_t)M.cols, (uint64_t)M.rows, 16); };
@@ -1630,21 +1787,28 @@ int setup_train(mlp_handle *h) {
     t.dz[l] = h->dZ[l].map;
     t.dzt[l] = h->dZt[l].map;
     if (!rc) rc = slices(&t.ht[l], h->Ht[l]);
+    if (!rc) rc = slices(&t.h16[l], h->H[l]);
+    if (!rc) rc = slices(&t.dz16[l], h->dZ[l]);
+    if (!rc) rc = slices(&t.dzt16[l], h->dZt[l]);
   }
+  if (!rc) rc = slices(&t.dy16, h->dY);
   t.ht_last = h->Ht[L - 2].map;
   t.dy = h->dY.map;
   t.dyt = h->dYt.map;
   if (rc) return rc;
-  OTF_CUDA(cudaMalloc(&h->loss_part, sizeof(double) * (h->cap / kBM)));
+  if (!h->loss_part) OTF_CUDA(cudaMalloc(&h->loss_part, sizeof(double) * (h->cap / kBM)));
+  if (!h->train_state) OTF_CUDA(cudaMalloc(&h->train_state, sizeof(float) * kTrainCtas * 2 * kMaxLayers * 3 * 256 * 8));
   OTF_CUDA(cudaFuncSetAttribute(k_train_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTrainSmem));
+  h->train_ready = true;
   return MD_OK;
 }
 
-// The steps of one epoch: nb batches of the prepared inputs behind maps x, xt
+// The steps of one epoch: nb batches of the prepared inputs behind maps x, x16, xt
 // and targets Ts; corr: their bias corrections (device).
-int train_epoch(mlp_handle *h, const Mat &Xs, const CUtensorMap &xt, const float *Ts, int64_t nb, const float2 *corr) {
+int train_epoch(mlp_handle *h, const Mat &Xs, const CUtensorMap &x16, const CUtensorMap &xt, const float *Ts, int64_t nb, const float2 *corr) {
   TrainMaps tm = h->trm;
   tm.x = Xs.map;
+  tm.x16 = x16;
   tm.xt = xt;
   TrainArgs a{};
   a.L = h->L;
@@ -1666,6 +1830,9 @@ int train_epoch(mlp_handle *h, const Mat &Xs, const CUtensorMap &xt, const float
   a.dYt = h->dYt.p;
   a.Ts = Ts;
   a.part = h->loss_part;
+  a.state = h->train_state;
+  a.inv = 1.0 / ((double)h->cap * h->p.n_out);
+  a.gscale = (float)(2.0 * a.inv);
   a.loss = h->loss;
   a.acc_scale = 1.0 / (double)nb;  // the loss slot adds up to the epoch's mean
   a.err = h->err;
@@ -1763,7 +1930,6 @@ int create_impl(mlp_handle *h) {
   OTF_CUDA(cudaMallocHost(&h->err_host, sizeof(unsigned)));
   *h->err_host = 0u;
   OTF_CUDA(cudaDeviceSynchronize());
-  if (int rt = setup_train(h)) return rt;
   return setup_fused(h);
 }
 
@@ -2065,14 +2231,16 @@ int mlp_train(mlp_handle *h, const float *X, const float *T, int64_t rows, int32
   int64_t *dperm = nullptr;
   double *dloss = nullptr;
   float2 *dcorr = nullptr;  // [nb] bias corrections of an epoch's steps
-  CUtensorMap xt_map;
+  CUtensorMap x16_map, xt_map;
   const float *dX = nullptr, *dT = nullptr;
   std::vector<double> hist((size_t)epochs, 0.0);
-  int rc = to_device(h, X, rows * h->p.n_in, mem, &ox, &dX);
+  int rc = setup_train(h);
+  if (!rc) rc = to_device(h, X, rows * h->p.n_in, mem, &ox, &dX);
   if (!rc) rc = to_device(h, T, rows * h->p.n_out, mem, &ot, &dT);
   if (!rc) rc = mat_alloc(Xall, rows, h->k_in, kBM);
   if (!rc) rc = mat_alloc(Xs, nused, h->k_in, kBM);
   if (!rc) rc = mat_alloc(Xst, h->k_in, nused, (uint32_t)h->k_in);
+  if (!rc) rc = make_map(&x16_map, Xs.p, (uint64_t)Xs.cols, (uint64_t)Xs.rows, 16);
   if (!rc) rc = make_map(&xt_map, Xst.p, (uint64_t)Xst.cols, (uint64_t)Xst.rows, 16);
   auto cuda_ok = [&](cudaError_t e) {
     if (e != cudaSuccess && !rc) {
@@ -2123,7 +2291,7 @@ int mlp_train(mlp_handle *h, const float *X, const float *T, int64_t rows, int32
                                     (float)(1.0 - std::pow((double)h->p.beta2, (double)h->t)));
     }
     if (!cuda_ok(cudaMemcpyAsync(dcorr, corr.data(), sizeof(float2) * nb, cudaMemcpyHostToDevice, h->st))) break;
-    rc = train_epoch(h, Xs, xt_map, Ts, nb, dcorr);
+    rc = train_epoch(h, Xs, x16_map, xt_map, Ts, nb, dcorr);
     if (!rc) cuda_ok(cudaMemcpyAsync(dloss + e, h->loss, sizeof(double), cudaMemcpyDeviceToDevice, h->st));
     if (!rc) cuda_ok(cudaMemsetAsync(h->loss, 0, sizeof(double), h->st));
     if (!rc) cuda_ok(cudaStreamSynchronize(h->st));  // the host permutation buffer is reused next epoch

@@ -261,3 +261,22 @@ def test_training_steps_equal_layered_steps(pkg, n_in, depth, batch, batches):
     d = np.abs(a.get_flat() - b.get_flat())
     assert np.linalg.norm(d) <= 1e-5 * np.linalg.norm(b.get_flat())
     assert d.max() <= 2.01 * lr * batches
+
+
+@pytest.mark.parametrize("batch", [128, 256])
+def test_training_wait_timeout_is_an_error_status(pkg, batch):
+    """The cluster's pipeline waits run out as the layered kernel's do: the
+    call ends with MD_ETIMEOUT and the handle stays usable."""
+    X = synth.normal(81, 2 * batch * 132).reshape(2 * batch, 132).astype(np.float32)
+    T = synth.normal(82, 2 * batch * 2).reshape(2 * batch, 2).astype(np.float32)
+    net = pkg.MLP(132, 2, batch=batch)
+    start = net.get_flat()
+    net.set_wait_limit(0)
+    with pytest.raises(pkg.MdError) as ei:
+        net.train(X, T, 2)
+    assert ei.value.code == -5  # MD_ETIMEOUT
+    net.set_wait_limit(2_000_000_000)
+    net.set_flat(start)
+    again = pkg.MLP(132, 2, batch=batch)
+    assert np.array_equal(net.train(X, T, 2), again.train(X, T, 2))
+    assert np.array_equal(net.get_flat(), again.get_flat())
