@@ -543,6 +543,16 @@ int Correlator::create(const corr_params &p, cudaStream_t s, cudaStream_t zero_o
     dev.vec = (dev.gs % vw == 0) ? vw : 1;
     // two vectors per thread when the group splits evenly into them
     dev.vu = (dev.vec == vw && dev.gs % (2 * vw) == 0) ? 2 : 1;
+    // fewer series per thread while a push would leave SMs idle (one CTA each):
+    // two vectors of four per thread are six CTAs at 4,000 atoms, and a pass of
+    // eight pushes took 73 us (FP64 143), with one series per thread 55
+    // (FP64 87)
+    const auto ctas = [&] {
+      const int64_t per = (int64_t)kPushThreads * dev.vec * dev.vu;
+      return dev.ng * ((dev.gs + per - 1) / per);
+    };
+    if (dev.vu > 1 && ctas() < 152) dev.vu = 1;
+    if (dev.vec > 1 && ctas() < 152) dev.vec = 1;
     const int64_t per_block = (int64_t)kPushThreads * dev.vec * dev.vu;
     dev.nchunk = (int)((dev.gs + per_block - 1) / per_block);
   } else {
