@@ -552,7 +552,7 @@ class MLP:
         else:
             import torch
 
-            Y = torch.zeros((rows, self.n_out), dtype=torch.float32, device=X.device)
+            Y = torch.empty((rows, self.n_out), dtype=torch.float32, device=X.device)  # every value is written
             py = Y.data_ptr()
         _check(lib().mlp_forward(self._h, px, rows, py, mem))
         return Y
