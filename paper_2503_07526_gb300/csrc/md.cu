@@ -415,7 +415,14 @@ __device__ __forceinline__ void rb_scan(const Sys &d, int r) {
   const int seg = (nc3 + 31) / 32;
   const int c0 = min(nc3, warp * seg), c1 = min(nc3, c0 + seg);
   int part = 0;
-  for (int c = c0 + lane; c < c1; c += 32) part += count[c];
+  constexpr int kRows = 8;  // rows of 32 counts whose loads are in flight together
+  for (int b = c0; b < c1; b += 32 * kRows) {
+    int v[kRows];
+#pragma unroll
+    for (int k = 0; k < kRows; ++k) v[k] = b + 32 * k + lane < c1 ? count[b + 32 * k + lane] : 0;
+#pragma unroll
+    for (int k = 0; k < kRows; ++k) part += v[k];
+  }
   part = warp_sum(part);
   if (lane == 0) wsum[warp] = part;
   __syncthreads();
@@ -431,20 +438,25 @@ __device__ __forceinline__ void rb_scan(const Sys &d, int r) {
   }
   __syncthreads();
   int carry = (int)R.atom0 + wsum[warp];
-  for (int b = c0; b < c1; b += 32) {
-    const int c = b + lane;
-    const int v = c < c1 ? count[c] : 0;
-    int incl = v;
+  for (int b = c0; b < c1; b += 32 * kRows) {
+    int v[kRows];
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
+    for (int k = 0; k < kRows; ++k) v[k] = b + 32 * k + lane < c1 ? count[b + 32 * k + lane] : 0;
+#pragma unroll
+    for (int k = 0; k < kRows; ++k) {
+      const int c = b + 32 * k + lane;
+      int incl = v[k];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      if (c < c1) {
+        start[c] = carry + incl - v[k];
+        count[c] = 0;
+      }
+      carry += __shfl_sync(0xffffffffu, incl, 31);
     }
-    if (c < c1) {
-      start[c] = carry + incl - v;
-      count[c] = 0;
-    }
-    carry += __shfl_sync(0xffffffffu, incl, 31);
   }
   __syncthreads();  // wsum is reused by the next replica
 }
@@ -1476,10 +1488,23 @@ __device__ __forceinline__ float dist2(const float4 &a, const float4 &b) {
 // against the 27 window cells around its own (nine contiguous slot ranges
 // of three cells), 32 slots at a time.  The distance tests (groups of eight,
 // predicated) fill two bit masks, within r_list and within the close radius
-// r_close + skin, before anything is appended; the accepted slots are then
-// appended in warp-uniform loops (as many rounds as the lane with the most
-// entries needs), close entries first.  Entries leave as blocks of eight in
-// slot order, the last block of each segment padded with the dummy slot 0.
+// r_close + skin, before anything is appended.  Close entries (about ten per
+// atom) are appended at once, in warp-uniform rounds; the far mask of a batch
+// is kept in shared memory with its first slot, and the far entries of all
+// batches are taken off the masks at the end, one per lane and round.  Rounds
+// then follow the longest list of the warp (about a tenth above the mean)
+// instead of the longest batch, three times the mean: 1,228 ->
+// 1,064 us per build at 2,048,000 atoms (71 registers; held to 64 it took 1,242,
+// and CTAs walking over a batch's tiles instead of one each made its builds
+// half again as slow).  Entries leave
+// as blocks of eight in slot order, the last block of each segment padded with
+// the dummy slot 0.  A lane whose masks do not fit empties them on the way (all
+// lanes then do, in the same order of entries).
+constexpr int kFarWords = 24;  // far masks kept per thread (about 20 at a liquid's density)
+size_t build_smem(int wcap, int threads) {
+  return ((tile_smem(wcap, false) + 15) & ~(size_t)15) + (size_t)threads * kFarWords * 6;
+}
+
 __global__ void __launch_bounds__(kTileThreadsMax, 2) k_build_tile(Sys d, LJ<float> lj) {
   if (!any_rebuild(d)) return;
   const Tile tl = d.tiles[blockIdx.x];
@@ -1500,6 +1525,11 @@ __global__ void __launch_bounds__(kTileThreadsMax, 2) k_build_tile(Sys d, LJ<flo
   if (!ok) return;
   stage_coords<false>(d, W, whi, nullptr, cellof);
   const uint32_t wbase = (uint32_t)__cvta_generic_to_shared(whi);
+  // this thread's far masks and their first slots, one row of the CTA each
+  uint32_t *fmask = reinterpret_cast<uint32_t *>(cellof + ((d.wcap + kWinPad + 15) & ~15)) + threadIdx.x;
+  unsigned short *fslot =
+      reinterpret_cast<unsigned short *>(fmask - threadIdx.x + kFarWords * blockDim.x) + threadIdx.x;
+  const int T = blockDim.x;
   const int64_t n = d.n;
   const int maxb = d.maxnb >> 3;
   int t1;
@@ -1511,22 +1541,46 @@ __global__ void __launch_bounds__(kTileThreadsMax, 2) k_build_tile(Sys d, LJ<flo
     uint4 *far = d.tnb + i;
     uint4 *cl = d.tcl + i;
     uint32_t fw[4] = {0u, 0u, 0u, 0u}, cw[4] = {0u, 0u, 0u, 0u};
-    int nfar = 0, ncl = 0;
+    int nfar = 0, ncl = 0, kept = 0, nw = 0;  // far entries written / in the masks, masks kept
+    const unsigned act = __activemask();
+    bool early = false;  // masks emptied on the way (uniform over the warp)
     auto put_far = [&](uint32_t off) {
       push16(fw, off);
       if ((++nfar & 7) == 0 && (nfar >> 3) <= maxb)
         far[(int64_t)((nfar >> 3) - 1) * n] = make_uint4(fw[0], fw[1], fw[2], fw[3]);
+    };
+    // the next far entry off the masks (0 once they are empty)
+    int w = 0;
+    uint32_t m = 0u, at = 0u;
+    auto pop = [&]() -> uint32_t {
+      if (m == 0u && w < nw) {
+        m = fmask[w * T];
+        at = fslot[w * T];
+        ++w;
+      }
+      if (m == 0u) return 0u;
+      const uint32_t off = (at + (uint32_t)__ffs(m) - 1u) << 4;
+      m &= m - 1u;
+      return off;
+    };
+    auto empty_masks = [&]() {
+      const int most = __reduce_max_sync(act, kept);
+      for (int k = 0; k < most; ++k) {
+        const uint32_t off = pop();
+        if (off) put_far(off);
+      }
+      w = nw = kept = 0;
     };
     for (int row = 0; row < 9; ++row) {
       const int c = ((wz + row / 3 - 1) * W.WY + (wy + row % 3 - 1)) * W.WX + wx - 1;
       const int s1 = W.pre[c + 3];
       for (int s = W.pre[c]; s < s1; s += 32) {
         const uint32_t a0 = wbase + ((uint32_t)s << 4);
-        const int m = min(32, s1 - s);
+        const int ms = min(32, s1 - s);
         uint32_t am = 0u, cm = 0u;
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
-          if (8 * g < m) {
+          if (8 * g < ms) {
             uint32_t ga = 0u, gc = 0u;
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
@@ -1538,32 +1592,35 @@ __global__ void __launch_bounds__(kTileThreadsMax, 2) k_build_tile(Sys d, LJ<flo
             cm |= gc << (8 * g);
           }
         }
-        if (m < 32) am &= (1u << m) - 1u;
+        if (ms < 32) am &= (1u << ms) - 1u;
         const int self = wi - s;
         if (self >= 0 && self < 32) am &= ~(1u << self);
         cm &= am;
         uint32_t fm = am & ~cm;
-        const unsigned act = __activemask();
-        const int mc = __reduce_max_sync(act, __popc(cm));
+        const unsigned here = __activemask();
+        const int mc = __reduce_max_sync(here, __popc(cm));
         for (int k = 0; k < mc; ++k) {
           if (cm) {
-            const int b = __ffs(cm) - 1;
+            const int bit = __ffs(cm) - 1;
             cm &= cm - 1u;
             if (ncl < kMaxCloseT) {
-              push16(cw, (uint32_t)(s + b) << 4);
+              push16(cw, (uint32_t)(s + bit) << 4);
               if ((++ncl & 7) == 0) cl[(int64_t)((ncl >> 3) - 1) * n] = make_uint4(cw[0], cw[1], cw[2], cw[3]);
             } else {
-              fm |= 1u << b;  // beyond the close capacity: FP32 displacement
+              fm |= 1u << bit;  // beyond the close capacity: FP32 displacement
             }
           }
         }
-        const int mf = __reduce_max_sync(act, __popc(fm));
-        for (int k = 0; k < mf; ++k) {
-          if (fm) {
-            const int b = __ffs(fm) - 1;
-            fm &= fm - 1u;
-            put_far((uint32_t)(s + b) << 4);
+        if (fm) {
+          if (nw == kFarWords) {  // full: this lane empties its masks now
+            for (uint32_t off = pop(); off; off = pop()) put_far(off);
+            w = nw = kept = 0;
+            early = true;
           }
+          fmask[nw * T] = fm;
+          fslot[nw * T] = (unsigned short)s;
+          ++nw;
+          kept += __popc(fm);
         }
       }
     }
@@ -1572,7 +1629,22 @@ __global__ void __launch_bounds__(kTileThreadsMax, 2) k_build_tile(Sys d, LJ<flo
       for (int k = 0; k < pad; ++k) push16(cw, 0u);
       cl[(int64_t)(ncl >> 3) * n] = make_uint4(cw[0], cw[1], cw[2], cw[3]);
     }
-    while (nfar & 7) put_far(0u);
+    if (__any_sync(act, early)) {
+      empty_masks();
+      while (nfar & 7) put_far(0u);
+    } else {  // every lane at entry 0: the blocks fill in step
+      const int blocks = (kept + 7) >> 3, most = __reduce_max_sync(act, blocks);
+      for (int b = 0; b < most; ++b) {
+        uint32_t v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const uint32_t lo = pop();
+          v[k] = lo | (pop() << 16);
+        }
+        if (b < blocks && b < maxb) far[(int64_t)b * n] = make_uint4(v[0], v[1], v[2], v[3]);
+      }
+      nfar = blocks * 8;
+    }
     d.nnb[i] = list_count(d, nfar) | (ncl << 16);
   }
 }
@@ -2516,7 +2588,7 @@ int launch_rebuild(md_handle *h, cudaStream_t s) {
   }
   if (h->prm.pair_mode == MD_PAIR_VERLET) launch_build<TF>(h, s);
   if (h->prm.pair_mode == MD_PAIR_TILES)
-    k_build_tile<<<tile_grid(h), tile_cta(h), tile_smem(d.wcap, false), s>>>(d, lj_of<float>(h->prm));
+    k_build_tile<<<tile_grid(h), tile_cta(h), build_smem(d.wcap, tile_cta(h)), s>>>(d, lj_of<float>(h->prm));
   OTF_LAUNCH_CHECK();
   return MD_OK;
 }
@@ -3105,7 +3177,7 @@ int finish_tiles(md_handle *h, cudaStream_t st) {
   OTF_CUDA(cudaMemcpyAsync(h->d_tiles, h->tiles_host.data(), nt * sizeof(Tile), cudaMemcpyHostToDevice, st));
   OTF_CUDA(cudaMemsetAsync(d.trec, 0xff, nt * sizeof(TileWin), st));
   OTF_CUDA(cudaFuncSetAttribute(k_build_tile, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)tile_smem(d.wcap, false)));
+                                (int)build_smem(d.wcap, kTileThreadsMax)));
   OTF_CUDA(cudaFuncSetAttribute(k_pair_tile, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)tile_smem(d.wcap, true)));
   return MD_OK;
@@ -3124,7 +3196,7 @@ int autotune_tiles(md_handle *h) {
   const size_t nflags = (size_t)(h->nrep + 1) * sizeof(int);
   auto build = [&] {
     cudaMemsetAsync(h->d.rebuild, 1, nflags, h->stream);
-    k_build_tile<<<tile_grid(h), tile_cta(h), tile_smem(h->d.wcap, false), h->stream>>>(h->d, lj);
+    k_build_tile<<<tile_grid(h), tile_cta(h), build_smem(h->d.wcap, tile_cta(h)), h->stream>>>(h->d, lj);
   };
   float best = 1e30f;
   int best_k = 0, best_t = h->tile_threads;
