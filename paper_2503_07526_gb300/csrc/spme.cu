@@ -433,17 +433,17 @@ __global__ void __launch_bounds__(kRowThreads) k_spme_spread(SpmeAtoms a, MeshPl
         for (int j = 0; j < na; ++j) {
           T *p = mine + b.x;
           const bool on = z < N && b.y + 4 * u < N;
-          const T qz = qx * wz;
-          T add[V];
+          const T w = wz;
+          T c[V];
 #pragma unroll
-          for (int v = 0; v < V; ++v) add[v] = qz * wy[v];
+          for (int v = 0; v < V; ++v) c[v] = qx * wy[v];
           read(min(j + 1, na - 1));
           if (on) {
             T t[V];
 #pragma unroll
             for (int v = 0; v < V; ++v) t[v] = p[-2 * v * sp.row];
 #pragma unroll
-            for (int v = 0; v < V; ++v) p[-2 * v * sp.row] = t[v] + add[v];
+            for (int v = 0; v < V; ++v) p[-2 * v * sp.row] = fma(c[v], w, t[v]);
           }
           __syncwarp();  // the next atom's points may be other lanes'
         }
@@ -512,7 +512,11 @@ __global__ void k_spme_conv(typename Cplx<T>::type *G1, typename Cplx<T>::type *
 // derivatives [axis][0..2][kMaxOrder].
 //
 // The (phi, psi) pairs are multiplied as pairs: two FP32 operations per
-// instruction (f32x2) in the mixed form.
+// instruction (f32x2) in the mixed form.  That form also takes the pair `mid` of
+// one point of the stencil off every point first: the long waves hardly change
+// over a stencil, and every force and virial sum holds a derivative weight, whose
+// sum is zero, so only their rounding is lost (the energy, whose weights sum to
+// one, gets it back).
 template <typename T>
 struct Pair;
 template <>
@@ -531,6 +535,10 @@ struct Pair<float> {
   __device__ __forceinline__ void fma(Pair a, Pair b) {  // this += a b
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(v) : "l"(a.v), "l"(b.v));
   }
+  __device__ __forceinline__ void less(Pair a) {  // this -= a
+    const Pair m = both(-1.f);
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(v) : "l"(a.v), "l"(m.v));
+  }
   __device__ __forceinline__ float2 get() const {
     float2 x;
     asm("mov.b64 {%0, %1}, %2;" : "=f"(x.x), "=f"(x.y) : "l"(v));
@@ -546,11 +554,15 @@ struct Pair<double> {
     v.x = ::fma(a.v.x, b.v.x, v.x);
     v.y = ::fma(a.v.y, b.v.y, v.y);
   }
+  __device__ __forceinline__ void less(Pair a) {
+    v.x -= a.v.x;
+    v.y -= a.v.y;
+  }
   __device__ __forceinline__ double2 get() const { return v; }
 };
 
 template <typename T, int N, typename Fetch>
-__device__ __forceinline__ void gather_lane(const T *w, int z, Fetch fetch, T (&out)[16]) {
+__device__ __forceinline__ void gather_lane(const T *w, int z, Pair<T> mid, Fetch fetch, T (&out)[16]) {
   using P = Pair<T>;
   P wx[N], dx[N];
   T ex[N];
@@ -569,11 +581,11 @@ __device__ __forceinline__ void gather_lane(const T *w, int z, Fetch fetch, T (&
     T s2 = T(0);
 #pragma unroll
     for (int t0 = 0; t0 < N; ++t0) {
-      const typename Two<T>::type v = fetch(t0, t1);
-      const P pv = P::of(v);
+      P pv = P::of(fetch(t0, t1));
+      if (sizeof(T) == 4) pv.less(mid);
       c0.fma(wx[t0], pv);
       c1.fma(dx[t0], pv);
-      s2 += ex[t0] * v.y;
+      s2 += ex[t0] * pv.get().y;
     }
     const T wy = w[3 * kMaxOrder + t1], dy = w[4 * kMaxOrder + t1], ey = w[5 * kMaxOrder + t1];
     const P wy2 = P::both(wy), dy2 = P::both(dy);
@@ -688,23 +700,25 @@ __global__ void __launch_bounds__(kRowThreads, sizeof(T) == 4 ? 5 : 2)
           const bool put = h + grp < nb && z < 5;
           const T v0 = put ? *r0 : T(0), v1 = put ? *r1 : T(0);
           T acc[16];
+          T2 mid = {T(0), T(0)};  // (phi, psi) at a point of the stencil that the group's lanes share
           if (tiled) {
             const int plane = tl.ey * tl.ez;
             const T2 *p = tile + (bx - tl.ox) * plane + (by - tl.oy) * tl.ez + (bz - tl.oz);
-            gather_lane<T, N>(wb + j * kGatherPitch, z, [&](int t0, int t1) { return p[-(t0 * plane + t1 * tl.ez)]; },
-                              acc);
+            if (sizeof(T) == 4) mid = p[min(z, N - 1) - N / 2 - N / 2 * (plane + tl.ez)];
+            gather_lane<T, N>(wb + j * kGatherPitch, z, Pair<T>::of(mid),
+                              [&](int t0, int t1) { return p[-(t0 * plane + t1 * tl.ez)]; }, acc);
           } else {
             const int iz = wrap_near(bz, K);
-            gather_lane<T, N>(
-                wb + j * kGatherPitch, z,
-                [&](int t0, int t1) {
-                  const int64_t m = ((int64_t)wrap_near(bx - t0, K) * K + wrap_near(by - t1, K)) * K + iz;
-                  T2 v;
-                  v.x = phi[m];
-                  v.y = psi[m];
-                  return v;
-                },
-                acc);
+            const auto at = [&](int t0, int t1, int mz) {
+              const int64_t m = ((int64_t)wrap_near(bx - t0, K) * K + wrap_near(by - t1, K)) * K + mz;
+              T2 v;
+              v.x = phi[m];
+              v.y = psi[m];
+              return v;
+            };
+            if (sizeof(T) == 4) mid = at(N / 2, N / 2, wrap_near(bz + min(z, N - 1) - N / 2, K));
+            gather_lane<T, N>(wb + j * kGatherPitch, z, Pair<T>::of(mid),
+                              [&](int t0, int t1) { return at(t0, t1, iz); }, acc);
           }
           // the group's sums: lane z ends with values 2 z and 2 z + 1
 #pragma unroll
@@ -717,7 +731,9 @@ __global__ void __launch_bounds__(kRowThreads, sizeof(T) == 4 ? 5 : 2)
             }
           }
           const T q = sq[b0 + j];
-          const T er = T(0.5) * ke * q * __shfl_sync(0xffffffffu, acc[0], lane & 24);
+          T pot = __shfl_sync(0xffffffffu, acc[0], lane & 24);
+          if (sizeof(T) == 4) pot += mid.x;  // the weights sum to one
+          const T er = T(0.5) * ke * q * pot;
           if (put) {
             const T fq = -ke * q * kL, wq = cw * q;
             *r0 = v0 + (z == 0 ? er - self * q * q : (z == 1 ? fq * acc[0] : (z < 4 ? er : T(0)) + wq * acc[0]));
@@ -754,10 +770,11 @@ constexpr size_t kMaxSpmeSmem =
 static_assert(kMaxSpmeSmem + 8 * 1024 <= 227 * 1024, "tile, weights and static tables fit one CTA");
 
 // Chunk and tile sizes: the largest chunk of 128, 64 or 32 atoms that still
-// gives four CTAs per SM (128 atoms share a tile's halo: at 512,000 ions 10
-// tile points are flushed per mesh point, against 17 with 32 atoms; below
-// 78,000 atoms more CTAs count for more), whose expected tile of the gather
-// (the cells the chunk spans plus the spline's support) fits.
+// gives four CTAs per SM in FP64, one per two SMs in the mixed form, whose
+// expected tile of the gather (the cells the chunk spans plus the spline's
+// support) fits.  128 atoms share a tile's halo (at 512,000 ions 10 tile points
+// are flushed per mesh point, against 17 with 32 atoms); below 78,000 atoms more
+// CTAs count for more in FP64, whose pipe they spread the work over.
 void plan_chunks(const SpmeAtoms &a, int order, size_t ts, MeshPlan &g) {
   const double cells = (double)a.nc * a.nc * a.nc, apc = a.n / cells, e = a.edge * g.kl;
   double pts = 0.0, words = 0.0;
@@ -766,7 +783,7 @@ void plan_chunks(const SpmeAtoms &a, int order, size_t ts, MeshPlan &g) {
     const SpreadPitch sp((int)side, (int)side);
     pts = side * side * len;
     words = len * sp.plane;
-    if (g.chunk == 32 || (a.n >= (int64_t)608 * g.chunk && pts * 2 * ts <= kMaxTileBytes / 2)) break;
+    if (g.chunk == 32 || (a.n >= (int64_t)(ts == 8 ? 608 : 76) * g.chunk && pts * 2 * ts <= kMaxTileBytes / 2)) break;
   }
   g.cap = (int)std::min(pts, (double)(kMaxTileBytes / (2 * ts)));
   g.cap = (g.cap + 3) & ~3;
