@@ -1,0 +1,158 @@
+"""Sizes on both sides of the lines at which the kernels change how they split
+their work, against the FP64 oracle (Sec. 2.2, Sec. 2.3, Appendix B).
+
+Tolerances are those of the paths' own parity tests: FP64 1e-11 of the largest
+magnitude (only summation orders differ); mixed 2e-5 for forces and
+correlators, 1e-4 for the ionic per-particle energies and virials (sums of
+large cancelling FP32 terms)."""
+import numpy as np
+import pytest
+
+from paper_2503_07526_gb300 import synth
+from test_gpu_corr import compare, series
+from test_gpu_ionic import ALPHA, MASSES, reference, system  # noqa: F401 (fixture)
+from test_gpu_ionic import params as ionic_params
+from test_gpu_md import F_AT_RC, check_mixed_forces, jittered, params, rel
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2503_07526_gb300 as pkg
+
+    pkg.lib(build=True)
+    return pkg
+
+
+@pytest.mark.parametrize("skin", [0.05, 0.3])
+@pytest.mark.parametrize("L", [32.0, 41.7])
+def test_fp64_pairs_next_to_the_cutoff(pkg, oracle_mod, L, skin):
+    """Dimers whose separations lie 1e-9, 1e-7 and 1e-5 rc inside and outside
+    the cutoff, at every place of the box: the lists are selected in FP32 with
+    an error band, the cutoff itself is decided in FP64."""
+    k = np.arange(64)
+    at = (np.stack([k % 4, k // 4 % 4, k // 16]) + 0.5) * (L / 4) + 0.5 * (synth.uniform01(3, 192).reshape(3, 64) - 0.5)
+    u = synth.uniform01(4, 192).reshape(3, 64) - 0.5
+    off = np.array([1e-9, -1e-9, 1e-7, -1e-7, 1e-5, -1e-5])[k % 6]
+    b = at + u / np.sqrt((u ** 2).sum(0)) * 2.5 * (1.0 + off)
+    r = np.mod(np.concatenate([at, b], axis=1), L)
+    s = dict(n=128, L=L)
+    g = pkg.System(params(pkg, s, precision=pkg.MD_PREC_FP64, skin=skin), r, np.zeros_like(r))
+    got = g.particles()
+    F, e, W = oracle_mod.lj_forces(r, L, method="cells")
+    assert ((F ** 2).sum(0) > 0).sum() == 2 * (off < 0).sum()  # half of the dimers interact
+    assert np.array_equal((got["F"] ** 2).sum(0) > 0, (F ** 2).sum(0) > 0)
+    assert rel(got["F"], F) <= 1e-11
+    assert np.abs(got["epot"] - e).max() <= 1e-11 * 2.5 * abs(F_AT_RC)
+    assert rel(got["W"], W) <= 1e-11
+
+
+@pytest.mark.parametrize("cells", [3, 16, 17, 18, 25, 27])
+@pytest.mark.parametrize("kind", ["fp64", "tiles"])
+def test_forces_and_reduction_over_sizes(pkg, oracle_mod, cells, kind):
+    """108 atoms; 16,384 and 19,652 (the sort within one cluster ends at the
+    first; the list build's warps per chunk and the tiles' CTAs change about
+    there); 23,328, 62,500 and 78,732 (10, 15 and 16 cells per side: tiles three
+    or two cells wide): forces, energies, virials and the reduction after two
+    steps, at the GPU's own positions."""
+    s = jittered(cells, seed=cells, rho=0.8442 if cells > 3 else 0.15)
+    if kind == "tiles":
+        if cells == 3:
+            s = jittered(5, seed=cells, rho=0.7)  # the tile path takes 3 cells per side at least
+        p = params(pkg, s, precision=pkg.MD_PREC_MIXED, pair_mode=pkg.MD_PAIR_TILES)
+    else:
+        p = params(pkg, s, precision=pkg.MD_PREC_FP64)
+    g = pkg.System(p, s["r"], s["v"])
+    g.step(2)
+    got, obs = g.particles(), g.observables()
+    F, e, W = oracle_mod.lj_forces(got["r"], s["L"], method="cells")
+    if kind == "fp64":
+        assert rel(got["F"], F) <= 1e-11
+        assert rel(got["epot"], e) <= 1e-11
+        assert rel(got["W"], W) <= 1e-11
+    else:
+        check_mixed_forces(got["F"], F, got["r"], s["L"], oracle_mod)
+    want = oracle_mod.observables(s["L"] ** 3, np.ones(s["n"]), got["v"], got["epot"], got["W"])
+    assert obs["U"] == pytest.approx(want[0], rel=1e-10)
+    assert rel(obs["sigma"], want[3:9]) <= 1e-10
+    assert rel(obs["q"], want[9:12]) <= 1e-10
+
+
+@pytest.mark.parametrize("kind", ["fp64", "tiles"])
+def test_replicas_of_unlike_size_equal_replicas_run_alone(pkg, kind):
+    """2,048 + 19,652 + 500 atoms in one handle: together they take the sort of
+    several launches and the scan per replica, alone the small ones take the
+    cluster's; the tile path agrees bit for bit, FP64 within summation order."""
+    reps = []
+    for k, (cells, rho) in enumerate(((8, 0.8), (17, 0.8442), (5, 0.7))):
+        t = jittered(cells, seed=60 + k, rho=rho, T=1.2, amp=0.15)
+        reps.append(dict(r=t["r"], v=t["v"], box=t["L"], n=t["n"]))
+    kw = dict(precision=pkg.MD_PREC_FP64) if kind == "fp64" else dict(precision=pkg.MD_PREC_MIXED, pair_mode=pkg.MD_PAIR_TILES)
+    kw.update(skin=0.2, stress=(6, 16, 2, 1), heatflux=(6, 16, 2, 1), vacf=None)
+    b = pkg.System(pkg.make_params(1, 1.0, **kw), replicas=reps)
+    b.step(20)
+    got, a0 = b.particles(), 0
+    for rp in reps:
+        alone = pkg.System(pkg.make_params(rp["n"], rp["box"], **kw), rp["r"], rp["v"])
+        alone.step(20)
+        want = alone.particles()
+        for key in ("r", "v", "F", "W"):
+            x = got[key][..., a0:a0 + rp["n"]]
+            assert np.array_equal(x, want[key]) if kind == "tiles" else rel(x, want[key]) <= 1e-13, key
+        a0 += rp["n"]
+
+
+_MESH = {}
+
+
+@pytest.mark.parametrize("precision,copies,order", [(0, 1, 4), (0, 2, 6), (0, 3, 8), (0, 4, 6),
+                                                    (1, 1, 6), (1, 2, 4), (1, 3, 8), (1, 4, 4)])
+def test_ionic_sizes_and_orders_match_oracle(pkg, system, precision, copies, order):  # noqa: F811
+    """1,728 to 110,592 ions: 32, 64 and 128 ions per chunk of the spread and
+    gather, spline orders 4, 6 and 8.  The larger systems are the small one
+    copied side by side on a mesh as many times finer, whose forces, energies
+    and virials are the small one's."""
+    from oracle import ewald
+
+    s = system
+    if order not in _MESH:
+        q = np.where(s["types"] == 0, 1.0, -1.0)
+        r = np.mod(s["r"], s["L"])
+        base = reference(s, 16)  # real-space and self terms; its mesh terms are exchanged for this order's
+        F8, E8, W8, _, _ = ewald.spme_reciprocal(r, q, s["L"], alpha=ALPHA, K=16, order=8)
+        Fk, Ek, Wk, _, _ = ewald.spme_reciprocal(r, q, s["L"], alpha=ALPHA, K=16, order=order)
+        _MESH[order] = dict(F=base["F"] - F8 + Fk, epot=base["epot"] - E8 + Ek, W=base["W"] - W8 + Wk)
+    ref, c = _MESH[order], copies
+    shift = s["L"] * np.stack(np.meshgrid(*[np.arange(c)] * 3, indexing="ij")).reshape(3, -1).astype(float)
+    r = (np.mod(s["r"], s["L"])[:, None, :] + shift[:, :, None]).reshape(3, -1)
+    big = dict(n=s["n"] * c ** 3, L=s["L"] * c)
+    p = ionic_params(pkg, big, precision, mesh=16 * c)
+    p.order = order
+    g = pkg.System(p, r, np.tile(s["v"], (1, c ** 3)), types=np.tile(s["types"], c ** 3))
+    got = g.particles()
+    g.close()
+    for key, t in (("F", 1e-11 if precision == 0 else 2e-5), ("epot", 1e-11 if precision == 0 else 1e-4),
+                   ("W", 1e-11 if precision == 0 else 1e-4)):
+        want = np.tile(ref[key], (1, c ** 3) if ref[key].ndim == 2 else c ** 3)
+        assert rel(got[key], want) <= t, key
+
+
+@pytest.mark.parametrize("b,p,m,ns,gs,prec,S", [
+    (4, 16, 2, 4864, 2432, 0, 100), (4, 16, 2, 4865, 973, 0, 100), (3, 32, 2, 4864, 1216, 1, 90),
+    (3, 32, 4, 4866, 811, 1, 90), (2, 16, 2, 300002, 150001, 1, 40), (2, 16, 2, 600000, 200000, 1, 40),
+    (2, 8, 2, 300000, 100000, 0, 24)])
+def test_corr_push_over_series_counts(pkg, oracle_mod, b, p, m, ns, gs, prec, S):
+    """A warp per series up to 4,864 series, a thread per one, two or four
+    series above (by the count and its divisibility)."""
+    x = series(ns, S, seed=ns)
+    g = pkg.Corr.create(b, p, m, ns, gs, False, prec)
+    o = oracle_mod.Corr(b, p, m, ns, gs, False)
+    for t in range(S):
+        g.push(x[t])
+        o.push(x[t])
+    compare(pkg, g, o, ns // gs, prec)
+    g.close()
