@@ -89,7 +89,7 @@ extern "C" {
 #define MD_PAIR_CELLS 1  /* direct link-cell evaluation every step */
 #define MD_PAIR_TILES 2  /* mixed-precision Lennard-Jones only: Verlet lists
                             (same skin rule) over tiles of at most 3 x 2 x 2
-                            cells (3 x 3 x 2 in small replicas); each tile's CTA stages the tile and its
+                            cells; each tile's CTA stages the tile and its
                             one-cell shell in shared memory, in the tile's own
                             frame, and the lists hold 16-bit offsets into that
                             window.  md_init returns MD_EINVAL when the
@@ -189,10 +189,8 @@ typedef struct {
   int64_t tiles;            /* MD_PAIR_TILES: tiles (CTAs of the pair kernel); else 0 */
   int32_t window_capacity;  /* MD_PAIR_TILES: shared-memory window slots per tile */
   int32_t tile_threads;     /* MD_PAIR_TILES: threads per tile CTA */
-  int32_t tile_extent[3];   /* MD_PAIR_TILES: the tiling's extent in cells along x, y, z
-                               (3 2 2 unless the autotuner picked another tiling; 3 2 2
-                               takes three cells along y in replicas of at most 15 cells
-                               per side) */
+  int32_t tile_extent[3];   /* MD_PAIR_TILES: largest tile extent in cells along x, y, z
+                               (3 2 2 unless the autotuner picked another tiling) */
 } md_config;
 
 /* Observables of the last completed step (Sec. 2.3). */

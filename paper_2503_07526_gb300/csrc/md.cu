@@ -3094,27 +3094,6 @@ void use_plan_host(md_handle *h, int k, int threads) {
   h->tile_threads = threads;
 }
 
-// Window slots that a tile of win_cells window cells may need: 1.2 times the
-// replica's mean density, or at least one atom per sigma^3, plus 64 slots.
-double window_need(const md_params &p, const Rep &R, int64_t n, double win_cells) {
-  const double apc = n / ((double)R.nc * R.nc * R.nc);
-  return win_cells * std::max(1.2 * apc, R.edge * R.edge * R.edge / (p.sigma * p.sigma * p.sigma)) + 64.0;
-}
-
-// Cells along y of the default tiling's tiles: 3 instead of 2 in replicas of at
-// most 15 cells per side whose wider windows fit the capacity.  Two-cell
-// segments of an odd side leave one-cell ones, whose windows are staged for a
-// third of the atoms, and of 500 to 32,000 atoms most of a tile's window is
-// shell: the 256-replica ensemble takes 16.6 ms per 20 steps instead of 18.6
-// (17.5 with the wider tiles on odd sides alone), single boxes the same time,
-// and at 2,048,000 atoms the two tilings differ by 1 %.  A function of the
-// replica alone, so that a batch computes each replica as it would alone.
-int default_tile_y(const md_params &p, const Rep &R, int64_t n, const int ext[3]) {
-  if (ext[0] != kTileExt[0] || ext[1] != kTileExt[1] || ext[2] != kTileExt[2] || R.nc > 15) return ext[1];
-  const int cap = p.window_slots > 0 ? p.window_slots : kWinMaxSlots;
-  return window_need(p, R, n, 5.0 * 5.0 * 4.0) <= cap ? 3 : ext[1];
-}
-
 int plan_tiles(const md_handle *h, const md_replica *reps, int count, const int ext[3], TilePlan &out) {
   const md_params &p = h->prm;
   out = TilePlan{};
@@ -3122,8 +3101,7 @@ int plan_tiles(const md_handle *h, const md_replica *reps, int count, const int 
   double need = 0.0, mean_win = 0.0, mean_tile = 0.0;
   for (int k = 0; k < count; ++k) {
     const Rep &R = h->reps[k];
-    const int ey = default_tile_y(p, R, reps[k].n, ext);
-    const auto sx = tile_segments(R.nc, ext[0]), sy = tile_segments(R.nc, ey), sz = tile_segments(R.nc, ext[2]);
+    const auto sx = tile_segments(R.nc, ext[0]), sy = tile_segments(R.nc, ext[1]), sz = tile_segments(R.nc, ext[2]);
     int mx = 0, my = 0, mz = 0;
     for (const auto &z : sz)
       for (const auto &y : sy)
@@ -3141,9 +3119,11 @@ int plan_tiles(const md_handle *h, const md_replica *reps, int count, const int 
           my = std::max(my, y.second);
           mz = std::max(mz, z.second);
         }
+    const double cell_vol = R.edge * R.edge * R.edge;
     const double apc = reps[k].n / ((double)R.nc * R.nc * R.nc);
+    const double s3 = p.sigma * p.sigma * p.sigma;
     const double win_cells = (double)(mx + 2) * (my + 2) * (mz + 2);
-    need = std::max(need, window_need(p, R, reps[k].n, win_cells));
+    need = std::max(need, win_cells * std::max(1.2 * apc, cell_vol / s3) + 64.0);
     mean_win = std::max(mean_win, win_cells * apc + 1.0);
     mean_tile = std::max(mean_tile, (double)mx * my * mz * apc);
   }
