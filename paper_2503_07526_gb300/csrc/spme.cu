@@ -470,35 +470,51 @@ __global__ void k_spme_unfix(const unsigned long long *Qi, T *Qr, int64_t total)
   }
 }
 
-// The two convolutions on the half spectrum [K][K][K/2+1].
-template <typename T>
-__global__ void k_spme_conv(typename Cplx<T>::type *G1, typename Cplx<T>::type *G2, const T *bmod, int K, T invL,
-                            T pa2, T cpre) {
+// The factors of both convolutions at mode e of the half spectrum
+// [K][K][K/2+1]; zero at the origin.
+__device__ __forceinline__ double2 conv_factors(int64_t e, int K, const double *bmod, double invL, double pa2,
+                                                double cpre) {
   const int kh = K / 2 + 1;
-  const int64_t total = (int64_t)K * K * kh;
+  const int iz = (int)(e % kh);
+  const int iy = (int)((e / kh) % K);
+  const int ix = (int)(e / ((int64_t)kh * K));
+  const double mx = (ix <= K / 2 ? ix : ix - K) * invL;
+  const double my = (iy <= K / 2 ? iy : iy - K) * invL;
+  const double mz = iz * invL;
+  const double m2 = mx * mx + my * my + mz * mz;
+  if (m2 == 0.0) return make_double2(0.0, 0.0);
+  const double t = pa2 * m2;
+  const double bc = bmod[ix] * bmod[iy] * bmod[iz] * exp(-t) / m2 * cpre;
+  return make_double2(bc, bc * 2.0 * (1.0 + t) / m2);
+}
+
+// The mixed form's factors, rounded once from FP64 when the plan is made: formed
+// in FP32 on every step, each carried the rounding of its exponent (3e-7 and
+// more of the factor) into every virial alike.
+__global__ void k_spme_factors(float2 *fac, int64_t total, int K, const double *bmod, double invL, double pa2,
+                               double cpre) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int iz = (int)(e % kh);
-    const int iy = (int)((e / kh) % K);
-    const int ix = (int)(e / ((int64_t)kh * K));
-    const T mx = (ix <= K / 2 ? ix : ix - K) * invL;
-    const T my = (iy <= K / 2 ? iy : iy - K) * invL;
-    const T mz = iz * invL;
-    const T m2 = mx * mx + my * my + mz * mz;
-    typename Cplx<T>::type g = G1[e];
-    if (m2 == T(0)) {
-      g.x = g.y = T(0);
-      G1[e] = g;
-      G2[e] = g;
-      continue;
-    }
-    const T t = pa2 * m2;
-    const T bc = bmod[ix] * bmod[iy] * bmod[iz] * exp(-t) / m2 * cpre;
-    const T bh = bc * T(2) * (T(1) + t) / m2;
-    typename Cplx<T>::type a = g, b = g;
-    a.x *= bc;
-    a.y *= bc;
-    b.x *= bh;
-    b.y *= bh;
+    const double2 f = conv_factors(e, K, bmod, invL, pa2, cpre);
+    fac[e] = make_float2((float)f.x, (float)f.y);
+  }
+}
+
+// The two convolutions on the half spectrum.
+template <typename T>
+__global__ void k_spme_conv(typename Cplx<T>::type *G1, typename Cplx<T>::type *G2, const float2 *fac,
+                            const double *bmod, int K, double invL, double pa2, double cpre) {
+  const int64_t total = (int64_t)K * K * (K / 2 + 1);
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+    typename Two<T>::type f;
+    if constexpr (std::is_same<T, double>::value)
+      f = conv_factors(e, K, bmod, invL, pa2, cpre);
+    else
+      f = fac[e];
+    typename Cplx<T>::type a = G1[e], b = a;
+    a.x *= f.x;
+    a.y *= f.x;
+    b.x *= f.y;
+    b.y *= f.y;
     G1[e] = a;
     G2[e] = b;
   }
@@ -815,12 +831,13 @@ int Spme::create(const SpmeParams &p, bool fp64, cudaStream_t st) {
   psi_ = static_cast<char *>(phi_) + ts * K3;
   OTF_CUDA(cudaMalloc(&G1_, 4 * ts * KH));
   G2_ = static_cast<char *>(G1_) + 2 * ts * KH;
-  OTF_CUDA(cudaMalloc(&bmod_, ts * K));
-  if (fp64) {
-    OTF_CUDA(cudaMemcpy(bmod_, bm.data(), sizeof(double) * K, cudaMemcpyHostToDevice));
-  } else {
-    std::vector<float> bf(bm.begin(), bm.end());
-    OTF_CUDA(cudaMemcpy(bmod_, bf.data(), sizeof(float) * K, cudaMemcpyHostToDevice));
+  OTF_CUDA(cudaMalloc(&bmod_, sizeof(double) * K));
+  OTF_CUDA(cudaMemcpy(bmod_, bm.data(), sizeof(double) * K, cudaMemcpyHostToDevice));
+  if (!fp64) {
+    OTF_CUDA(cudaMalloc(&fac_, sizeof(float2) * KH));
+    k_spme_factors<<<grid_of(KH), 256, 0, st>>>(fac_, KH, K, bmod_, 1.0 / p.L, kPi * kPi / (p.alpha * p.alpha),
+                                                1.0 / (kPi * p.L * p.L * p.L));
+    OTF_LAUNCH_CHECK();
   }
   int rc = cufft_ok(cufftPlan3d(&fwd_, K, K, K, fp64 ? CUFFT_D2Z : CUFFT_R2C), "cufftPlan3d (forward)");
   int dims[3] = {K, K, K};
@@ -840,10 +857,12 @@ void Spme::destroy() {
     cufftDestroy(inv_);
     plans_ = false;
   }
-  for (void *q : {(void *)Qi_, Qr_, phi_, G1_, bmod_})
+  for (void *q : {(void *)Qi_, Qr_, phi_, G1_, (void *)bmod_, (void *)fac_})
     if (q) cudaFree(q);
   Qi_ = nullptr;
-  Qr_ = phi_ = psi_ = G1_ = G2_ = bmod_ = nullptr;
+  Qr_ = phi_ = psi_ = G1_ = G2_ = nullptr;
+  bmod_ = nullptr;
+  fac_ = nullptr;
 }
 
 template <typename T>
@@ -898,8 +917,8 @@ int Spme::run_t(const SpmeAtoms &a, T *F, T *epot, T *W, cudaStream_t st) {
   if (rc) return rc;
   const double V = p_.L * p_.L * p_.L;
   k_spme_conv<T><<<grid_of((int64_t)K * K * (K / 2 + 1)), 256, 0, st>>>(
-      static_cast<C *>(G1_), static_cast<C *>(G2_), static_cast<const T *>(bmod_), K, (T)(1.0 / p_.L),
-      (T)(kPi * kPi / (p_.alpha * p_.alpha)), (T)(1.0 / (kPi * V)));
+      static_cast<C *>(G1_), static_cast<C *>(G2_), fac_, bmod_, K, 1.0 / p_.L, kPi * kPi / (p_.alpha * p_.alpha),
+      1.0 / (kPi * V));
   OTF_LAUNCH_CHECK();
   if constexpr (std::is_same<T, double>::value) {
     rc = cufft_ok(cufftExecZ2D(inv_, static_cast<C *>(G1_), static_cast<double *>(phi_)), "cufftExecZ2D");

@@ -51,7 +51,8 @@ class Spme {
   void *Qr_ = nullptr;                // real mesh [K^3]
   void *G1_ = nullptr, *G2_ = nullptr;  // half spectra [K][K][K/2+1], one allocation (G1_)
   void *phi_ = nullptr, *psi_ = nullptr;  // convolved meshes [K^3], one allocation (phi_)
-  void *bmod_ = nullptr;              // |b(m)|^2 [K]
+  double *bmod_ = nullptr;            // |b(m)|^2 [K]
+  float2 *fac_ = nullptr;             // convolution factors of the mixed form [K][K][K/2+1]
   cufftHandle fwd_ = 0, inv_ = 0;
   bool plans_ = false;
   bool attr_ = false;  // shared-memory limits raised for the tile kernels

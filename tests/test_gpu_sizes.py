@@ -56,8 +56,8 @@ def test_fp64_pairs_next_to_the_cutoff(pkg, oracle_mod, L, skin):
 def test_forces_and_reduction_over_sizes(pkg, oracle_mod, cells, kind):
     """108 atoms; 16,384 and 19,652 (the sort within one cluster ends at the
     first; the list build's warps per chunk and the tiles' CTAs change about
-    there); 23,328, 62,500 and 78,732 (10, 15 and 16 cells per side: tiles three
-    or two cells wide): forces, energies, virials and the reduction after two
+    there); 23,328, 62,500 and 78,732 (10, 15 and 16 cells per side, segments
+    of unlike length): forces, energies, virials and the reduction after two
     steps, at the GPU's own positions."""
     s = jittered(cells, seed=cells, rho=0.8442 if cells > 3 else 0.15)
     if kind == "tiles":
