@@ -88,16 +88,6 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
       : "memory");
 }
-// The same into the same place of every CTA of the cluster in the mask, each
-// CTA's barrier counting its copy.
-__device__ __forceinline__ void tma_load_2d_all(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar,
-                                                uint16_t mask) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1, {%2, "
-      "%3}], [%4], %5;" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar), "h"(mask)
-      : "memory");
-}
 __device__ __forceinline__ void tmem_alloc(uint32_t slot, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot), "r"(ncols) : "memory");
   asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -844,7 +834,7 @@ __global__ void k_cast_weights(const float *__restrict__ w, AdamTable tab) {
 // thread per row).  Here every product is cut into column slices over the
 // eight CTAs, and the phases of a step (one per layer forward, one per layer
 // back, the last weight gradient with Adam) are separated by cluster barriers:
-// 38 us per step (train_3584: 12.95 -> 2.86 ms for 56 steps with the call's
+// 39 us per step (train_3584: 12.95 -> 2.80 ms for 56 steps with the call's
 // set-up).  Operands go through global memory (L2) in the same matrices as the
 // layered kernels use and come back by TMA, the writers fencing the async proxy
 // before each barrier; each weight gradient's product runs beside the next
@@ -863,7 +853,6 @@ constexpr size_t kTrainSmem = 1024 + (size_t)kTrainStages * kStageBytes;
 struct TrainMaps {
   CUtensorMap x, xt;                     // this epoch's inputs: boxes of 128 rows; transposed, boxes of 16
   CUtensorMap h[kMaxLayers], dz[kMaxLayers], dzt[kMaxLayers], dy, ht_last;  // A operands, boxes of 128 rows
-  CUtensorMap x16, h16[kMaxLayers], dz16[kMaxLayers], dzt16[kMaxLayers], dy16;  // the same in boxes of 16 rows
   CUtensorMap w[kMaxLayers], wt[kMaxLayers], ht[kMaxLayers], dyt;           // B operands, boxes of 16 rows
 };
 struct TrainArgs {
@@ -921,10 +910,9 @@ __device__ __forceinline__ uint4 pack8(const bf16 (&b)[8]) {
 // One product of a phase: D [128 x N] at TMEM column col = A rows [arow, +128)
 // x B rows [brow, +N) over K columns from ak and bk; bar: arrives when it and
 // every product before it are done.
-// B rows come 16 at a time, bstep apart.  shared: the map of A in boxes of 16
-// rows when every CTA of the cluster takes the same A in this phase.
+// B rows come 16 at a time, bstep apart.
 struct TrainJob {
-  const CUtensorMap *ma, *mb, *shared;
+  const CUtensorMap *ma, *mb;
   int arow, ak, brow, bstep, bk, K, N, col;
   uint32_t bar;
 };
@@ -951,12 +939,11 @@ __global__ void __cluster_dims__(kTrainCtas, 1, 1) __launch_bounds__(kTrainThrea
   if (tid == 0) {
     for (int s = 0; s < 2 * kTrainStages + 1 + kMaxLayers; ++s) mbar_init(smem_u32(&bars[s]), 1);
     dead = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");  // before the copies that count on them
   }
   if (warp == 0) tmem_alloc(smem_u32(&slot), 512);
   tc_fence_before();
   __syncthreads();
-  cluster_sync();  // every CTA's barriers are set up before another's copies count on them
   tc_fence_after();
   const uint32_t tmem = slot;
   const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16);
@@ -965,13 +952,6 @@ __global__ void __cluster_dims__(kTrainCtas, 1, 1) __launch_bounds__(kTrainThrea
   const int wsl = kBM / nsl, tiles = mt * nsl;
   const bool epi = warp < kEpiWarps, issuer = warp == kEpiWarps && lane == 0;
 
-  // With one 128-row tile per batch every CTA multiplies by the same A: each
-  // fetches an eighth of it for all (TMA multicast).  Eight CTAs fetching all
-  // of it took about 10 bytes per cycle and SM.  Every CTA then issues the same
-  // panels (some ignore a product's result), so their stages stay in step; a
-  // phase uses no stage twice and ends with its products done, so the cluster barrier between
-  // phases also says that every CTA's stages are free.
-  const bool multi = mt == 1;
   // issuer: panels issued and consumed so far (stage = count mod kTrainStages)
   uint32_t issued = 0, consumed = 0;
   // a phase's product (or two, the second's copies running ahead of the
@@ -995,12 +975,9 @@ __global__ void __cluster_dims__(kTrainCtas, 1, 1) __launch_bounds__(kTrainThrea
         const uint32_t fb = smem_u32(&bars[s]), sa = smem_u32(smem + s * kStageBytes);
         const int N = second ? j1.N : j0.N, ax = (second ? j1.ak : j0.ak) + p * kBK, ay = second ? j1.arow : j0.arow;
         const int bx = (second ? j1.bk : j0.bk) + p * kBK, by = second ? j1.brow : j0.brow, bs = second ? j1.bstep : j0.bstep;
-        const CUtensorMap *mb = second ? j1.mb : j0.mb, *ms = second ? j1.shared : j0.shared;
+        const CUtensorMap *mb = second ? j1.mb : j0.mb;
         mbar_expect_tx(fb, kPanelBytes + (uint32_t)N * 128u);
-        if (multi && ms)
-          tma_load_2d_all(sa + rank * 16u * 128u, ms, ax, ay + rank * 16, fb, (uint16_t)((1 << kTrainCtas) - 1));
-        else
-          tma_load_2d(sa, second ? j1.ma : j0.ma, ax, ay, fb);
+        tma_load_2d(sa, second ? j1.ma : j0.ma, ax, ay, fb);
         for (int r = 0, y = by; r < N; r += 16, y += bs) tma_load_2d(sa + kPanelBytes + r * 128u, mb, bx, y, fb);
         ++issued;
       }
@@ -1029,10 +1006,6 @@ __global__ void __cluster_dims__(kTrainCtas, 1, 1) __launch_bounds__(kTrainThrea
       if (!first) mma_commit(j0.bar);
     }
     if (nj > 1) mma_commit(j1.bar);
-    if (multi && consumed > 0) {
-      const uint32_t last = consumed - 1;
-      if (!mbar_wait_blocking(smem_u32(&bars[kTrainStages + last % kTrainStages]), (last / kTrainStages) & 1u)) dead = 1;
-    }
   };
   // epilogue and Adam warps: waits for a barrier's phase; uniform over a warp
   auto ready = [&](uint32_t bar, uint32_t parity) {
@@ -1152,8 +1125,7 @@ __global__ void __cluster_dims__(kTrainCtas, 1, 1) __launch_bounds__(kTrainThrea
       for (int t = rank; t < tiles; t += kTrainCtas) {
         const int m0 = (t / nsl) * kBM, n0 = (t % nsl) * wsl;
         if (issuer) {
-          const TrainJob j = TrainJob{l == 0 ? &tm.x : &tm.h[l - 1], &tm.w[l], l == 0 ? &tm.x16 : &tm.h16[l - 1],
-                             (l == 0 ? row0 : 0) + m0, 0, n0, 16, 0, a.in_k[l], wsl, 0, done_bar};
+          const TrainJob j{l == 0 ? &tm.x : &tm.h[l - 1], &tm.w[l], (l == 0 ? row0 : 0) + m0, 0, n0, 16, 0, a.in_k[l], wsl, 0, done_bar};
           run_jobs(j, j, 1);
         }
         if (epi && ready(done_bar, phase)) {
@@ -1176,13 +1148,12 @@ __global__ void __cluster_dims__(kTrainCtas, 1, 1) __launch_bounds__(kTrainThrea
       phase_end();
     }
     // output layer, loss and its gradient (tile t: rows of one CTA)
-    for (int t = rank; t < mt || (multi && t == rank); t += kTrainCtas) {
-      const bool mine = t < mt;
-      if (issuer) {  // with a shared A the others copy their part too
-        const TrainJob j{&tm.h[L - 2], &tm.w[L - 1], &tm.h16[L - 2], mine ? t * kBM : 0, 0, 0, 16, 0, a.in_k[L - 1], kOutPad, 0, done_bar};
+    for (int t = rank; t < mt; t += kTrainCtas) {
+      if (issuer) {
+        const TrainJob j{&tm.h[L - 2], &tm.w[L - 1], t * kBM, 0, 0, 16, 0, a.in_k[L - 1], kOutPad, 0, done_bar};
         run_jobs(j, j, 1);
       }
-      if (epi && mine) {
+      if (epi) {
         const int64_t m = (int64_t)t * kBM + row;
         float tgt[8];
 #pragma unroll
@@ -1231,14 +1202,12 @@ __global__ void __cluster_dims__(kTrainCtas, 1, 1) __launch_bounds__(kTrainThrea
         if (issuer) {
           TrainJob j{}, g{};
           if (mine)
-            j = TrainJob{top ? &tm.dy : &tm.dz[l + 1], &tm.wt[l + 1], top ? &tm.dy16 : &tm.dz16[l + 1], m0, 0, n0, 16, 0,
-                         top ? kOutPad : kBM, wsl, 0, done_bar};
-          const bool grad = !graded && (multi || has_slice(l + 1, 0));
+            j = TrainJob{top ? &tm.dy : &tm.dz[l + 1], &tm.wt[l + 1], m0, 0, n0, 16, 0, top ? kOutPad : kBM, wsl, 0, done_bar};
+          const bool grad = !graded && has_slice(l + 1, 0);
           if (top)
-            g = TrainJob{&tm.ht_last, &tm.dyt, &tm.ht[l], 0, 0, 0, 16, 0, a.cap, kOutPad, kGradCol + 32 * (l + 1), grad_bar(l + 1)};
+            g = TrainJob{&tm.ht_last, &tm.dyt, 0, 0, 0, 16, 0, a.cap, kOutPad, kGradCol + 32 * (l + 1), grad_bar(l + 1)};
           else
-            g = TrainJob{&tm.dzt[l + 1], &tm.ht[l], &tm.dzt16[l + 1], 0, 0, rank * 16, 16, 0, a.cap, 16, kGradCol + 32 * (l + 1),
-                         grad_bar(l + 1)};
+            g = TrainJob{&tm.dzt[l + 1], &tm.ht[l], 0, 0, rank * 16, 16, 0, a.cap, 16, kGradCol + 32 * (l + 1), grad_bar(l + 1)};
           if (mine)
             run_jobs(j, g, grad ? 2 : 1);
           else if (grad)
@@ -1274,12 +1243,9 @@ __global__ void __cluster_dims__(kTrainCtas, 1, 1) __launch_bounds__(kTrainThrea
       phase_end();
     }
     // the first layer's weight gradient, the biases, then the last two layers' Adam
-    if (issuer) {
-      // slices rank and rank + 8 of the inputs, as far as there are any; with a
-      // shared A every CTA takes its part in the copies
+    if (issuer && has_slice(0, 0)) {  // slices rank and rank + 8 of the inputs, as far as there are any
       const int N = has_slice(0, 1) ? 32 : 16;
-      const bool any = has_slice(0, 0);
-      const TrainJob j{&tm.dzt[0], &tm.xt, &tm.dzt16[0], 0, 0, any ? rank * 16 : 0, 16 * kTrainCtas, row0, a.cap, N, kGradCol, grad_bar(0)};
+      const TrainJob j{&tm.dzt[0], &tm.xt, 0, 0, rank * 16, 16 * kTrainCtas, row0, a.cap, N, kGradCol, grad_bar(0)};
       run_jobs(j, j, 1);
     } else if (warp > kEpiWarps && warp < kAdamWarp0) {
       // bias gradients: the rows of dZ^T summed as k_bias_grad does (the same
@@ -1348,7 +1314,6 @@ __global__ void __cluster_dims__(kTrainCtas, 1, 1) __launch_bounds__(kTrainThrea
   }
   tc_fence_before();
   __syncthreads();
-  cluster_sync();  // no copy of this CTA is on its way to another that has left
   if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
@@ -1788,11 +1753,7 @@ int setup_train(mlp_handle *h) {
     t.dz[l] = h->dZ[l].map;
     t.dzt[l] = h->dZt[l].map;
     if (!rc) rc = slices(&t.ht[l], h->Ht[l]);
-    if (!rc) rc = slices(&t.h16[l], h->H[l]);
-    if (!rc) rc = slices(&t.dz16[l], h->dZ[l]);
-    if (!rc) rc = slices(&t.dzt16[l], h->dZt[l]);
   }
-  if (!rc) rc = slices(&t.dy16, h->dY);
   t.ht_last = h->Ht[L - 2].map;
   t.dy = h->dY.map;
   t.dyt = h->dYt.map;
@@ -1804,12 +1765,11 @@ int setup_train(mlp_handle *h) {
   return MD_OK;
 }
 
-// The steps of one epoch: nb batches of the prepared inputs behind maps x, x16, xt
+// The steps of one epoch: nb batches of the prepared inputs Xs (transposed: map xt)
 // and targets Ts; corr: their bias corrections (device).
-int train_epoch(mlp_handle *h, const Mat &Xs, const CUtensorMap &x16, const CUtensorMap &xt, const float *Ts, int64_t nb, const float2 *corr) {
+int train_epoch(mlp_handle *h, const Mat &Xs, const CUtensorMap &xt, const float *Ts, int64_t nb, const float2 *corr) {
   TrainMaps tm = h->trm;
   tm.x = Xs.map;
-  tm.x16 = x16;
   tm.xt = xt;
   TrainArgs a{};
   a.L = h->L;
@@ -2236,7 +2196,7 @@ int mlp_train(mlp_handle *h, const float *X, const float *T, int64_t rows, int32
   int64_t *dperm = nullptr;
   double *dloss = nullptr;
   float2 *dcorr = nullptr;  // [nb] bias corrections of an epoch's steps
-  CUtensorMap x16_map, xt_map;
+  CUtensorMap xt_map;
   const float *dX = nullptr, *dT = nullptr;
   std::vector<double> hist((size_t)epochs, 0.0);
   int rc = setup_train(h);
@@ -2245,7 +2205,6 @@ int mlp_train(mlp_handle *h, const float *X, const float *T, int64_t rows, int32
   if (!rc) rc = mat_alloc(Xall, rows, h->k_in, kBM);
   if (!rc) rc = mat_alloc(Xs, nused, h->k_in, kBM);
   if (!rc) rc = mat_alloc(Xst, h->k_in, nused, (uint32_t)h->k_in);
-  if (!rc) rc = make_map(&x16_map, Xs.p, (uint64_t)Xs.cols, (uint64_t)Xs.rows, 16);
   if (!rc) rc = make_map(&xt_map, Xst.p, (uint64_t)Xst.cols, (uint64_t)Xst.rows, 16);
   auto cuda_ok = [&](cudaError_t e) {
     if (e != cudaSuccess && !rc) {
@@ -2296,7 +2255,7 @@ int mlp_train(mlp_handle *h, const float *X, const float *T, int64_t rows, int32
                                     (float)(1.0 - std::pow((double)h->p.beta2, (double)h->t)));
     }
     if (!cuda_ok(cudaMemcpyAsync(dcorr, corr.data(), sizeof(float2) * nb, cudaMemcpyHostToDevice, h->st))) break;
-    rc = train_epoch(h, Xs, x16_map, xt_map, Ts, nb, dcorr);
+    rc = train_epoch(h, Xs, xt_map, Ts, nb, dcorr);
     if (!rc) cuda_ok(cudaMemcpyAsync(dloss + e, h->loss, sizeof(double), cudaMemcpyDeviceToDevice, h->st));
     if (!rc) cuda_ok(cudaMemsetAsync(h->loss, 0, sizeof(double), h->st));
     if (!rc) cuda_ok(cudaStreamSynchronize(h->st));  // the host permutation buffer is reused next epoch
