@@ -2258,11 +2258,11 @@ int mlp_train(mlp_handle *h, const float *X, const float *T, int64_t rows, int32
     rc = train_epoch(h, Xs, xt_map, Ts, nb, dcorr);
     if (!rc) cuda_ok(cudaMemcpyAsync(dloss + e, h->loss, sizeof(double), cudaMemcpyDeviceToDevice, h->st));
     if (!rc) cuda_ok(cudaMemsetAsync(h->loss, 0, sizeof(double), h->st));
-    if (!rc) cuda_ok(cudaStreamSynchronize(h->st));  // the host permutation buffer is reused next epoch
+    // the host buffers are reused next epoch; an epoch whose waits gave up is the last
+    if (!rc) rc = check_err(h);
   }
   if (!rc && epochs > 0)
     cuda_ok(cudaMemcpyAsync(hist.data(), dloss, sizeof(double) * epochs, cudaMemcpyDeviceToHost, h->st));
-  if (!rc) rc = check_err(h);
   cudaStreamSynchronize(h->st);
   if (!rc && loss_per_epoch) std::memcpy(loss_per_epoch, hist.data(), sizeof(double) * epochs);
   mat_free(Xall);

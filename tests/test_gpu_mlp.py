@@ -280,3 +280,23 @@ def test_training_wait_timeout_is_an_error_status(pkg, batch):
     again = pkg.MLP(132, 2, batch=batch)
     assert np.array_equal(net.train(X, T, 2), again.train(X, T, 2))
     assert np.array_equal(net.get_flat(), again.get_flat())
+
+
+def test_training_stops_at_the_first_epoch_that_gives_up(pkg):
+    """Epochs after one whose waits gave up are not run: the step count, which
+    sets Adam's bias corrections, is the same after one epoch asked for and
+    after forty."""
+    X = synth.normal(91, 256 * 132).reshape(256, 132).astype(np.float32)
+    T = synth.normal(92, 256 * 2).reshape(256, 2).astype(np.float32)
+    got = []
+    for epochs in (1, 40):
+        net = pkg.MLP(132, 2, batch=128)
+        net.set_flat(np.linspace(-0.1, 0.1, net.nparams, dtype=np.float32))
+        net.set_wait_limit(0)
+        with pytest.raises(pkg.MdError) as ei:
+            net.train(X, T, epochs)
+        assert ei.value.code == -5  # MD_ETIMEOUT
+        net.adam_step(np.ones(net.nparams, dtype=np.float32))
+        got.append(net.get_flat())
+        net.close()
+    assert np.array_equal(got[0], got[1])
