@@ -3170,16 +3170,18 @@ int setup_tiles(md_handle *h, const md_replica *reps, int count) {
 // MD_PAIR_TILES, once the arrays are carved (and again for every tiling the
 // autotuner tries): the tile table uploaded, every record marked "no window"
 // (natoms = -1) until the next list build, and the kernels' shared-memory
-// limits set to the window size.
+// limits raised.  A limit belongs to the kernel, not to the handle, so every
+// handle sets the same one, that of the largest window: set to a handle's own
+// window, a second handle with a smaller one took the first one's launches away.
 int finish_tiles(md_handle *h, cudaStream_t st) {
   Sys &d = h->d;
   const size_t nt = h->tiles_host.size();
   OTF_CUDA(cudaMemcpyAsync(h->d_tiles, h->tiles_host.data(), nt * sizeof(Tile), cudaMemcpyHostToDevice, st));
   OTF_CUDA(cudaMemsetAsync(d.trec, 0xff, nt * sizeof(TileWin), st));
   OTF_CUDA(cudaFuncSetAttribute(k_build_tile, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)build_smem(d.wcap, kTileThreadsMax)));
+                                (int)build_smem(kWinMaxSlots, kTileThreadsMax)));
   OTF_CUDA(cudaFuncSetAttribute(k_pair_tile, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)tile_smem(d.wcap, true)));
+                                (int)tile_smem(kWinMaxSlots, true)));
   return MD_OK;
 }
 

@@ -222,3 +222,25 @@ def test_tiles_autotune_batch(pkg, oracle_mod):
         sl = slice(a0, a0 + rp["n"])
         a0 += rp["n"]
         check_particles({key: got[key][..., sl] for key in ("r", "F", "epot", "W")}, oracle_mod, rp["box"])
+
+
+@pytest.mark.parametrize("use_graph", [True, False])
+def test_windows_of_unlike_size_in_one_process(pkg, use_graph):
+    """A kernel's shared-memory limit holds for the whole process: a second
+    handle with a small window, made before the first one's first step, leaves
+    the first one's launches (and the graphs captured then) as they are alone."""
+    s, small = jittered(8, seed=5), jittered(5, seed=6, rho=0.1)
+    kw = dict(window_slots=4096, use_graph=use_graph)
+    alone = pkg.System(tiles(pkg, s, **kw), s["r"], s["v"])
+    alone.step(20)
+    want = alone.particles()
+    alone.close()
+    g = pkg.System(tiles(pkg, s, **kw), s["r"], s["v"])
+    other = pkg.System(tiles(pkg, small, window_slots=512, use_graph=use_graph), small["r"], small["v"])
+    g.step(20)
+    other.step(3)
+    got = g.particles()
+    for key in ("r", "v", "F", "W", "epot"):
+        assert np.array_equal(got[key], want[key]), key
+    other.close()
+    g.close()
