@@ -581,9 +581,13 @@ __global__ void __launch_bounds__(kCellWarps * 32) k_rb_rank(Sys d) {
 // sixth of a 4,000-atom step; on a rebuild the phases are latency-bound and a
 // few SMs are enough.  Per sort at 4,000 atoms: 21 us mixed, 42 us FP64, the
 // separate kernels 29 and 32; one CTA instead of eight 46 and 132; at 37,000
-// atoms 66 against 32, so larger systems keep the separate kernels.
+// atoms 66 against 32, so larger systems keep the separate kernels.  So do
+// dilute ones, whose sort follows the cells (its last phase walks over them):
+// a step of 4,000 atoms at dt 0.005 takes, cluster / separate, 41 / 43 us with
+// 216 cells (FP64 52 / 53), 32 / 34 with 512 (44 / 43), 29 / 30 with 1,728
+// (44 / 38), 32 / 29 with 4,096 (52 / 38) and 69 / 30 with 110,592 (78 / 37).
 constexpr int kSortCtas = 8;
-constexpr int64_t kSortSmallAtoms = 16384;
+constexpr int64_t kSortSmallAtoms = 16384, kSortSmallCells = 1024;
 __device__ __forceinline__ void sort_sync() {
   asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
 }
@@ -2578,7 +2582,7 @@ template <typename TF>
 int launch_rebuild(md_handle *h, cudaStream_t s) {
   const Sys &d = h->d;
   KTimer tm(h, s, MD_K_REBUILD);
-  if (d.n <= kSortSmallAtoms) {
+  if (d.n <= kSortSmallAtoms && d.ncell <= kSortSmallCells) {
     k_rb_small<TF><<<kSortCtas, 1024, 0, s>>>(d);
   } else {
     k_rb_assign<TF><<<grid_for(d.n, kThreads), kThreads, 0, s>>>(d);

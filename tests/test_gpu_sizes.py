@@ -156,3 +156,58 @@ def test_corr_push_over_series_counts(pkg, oracle_mod, b, p, m, ns, gs, prec, S)
         o.push(x[t])
     compare(pkg, g, o, ns // gs, prec)
     g.close()
+
+
+def dilute(n, cells, seed):
+    """n atoms on a jittered cubic lattice in a box of `cells` cells per side."""
+    L = 2.8 * cells * 1.001
+    k = int(np.ceil(n ** (1.0 / 3.0) - 1e-9))
+    at = np.linspace(0, k ** 3 - 1, n).astype(np.int64)
+    r = (np.stack([at % k, at // k % k, at // (k * k)]) + 0.5) * (L / k)
+    r = r + 0.2 * (synth.uniform01(seed, 3 * n).reshape(3, n) - 0.5)
+    return dict(r=np.ascontiguousarray(np.mod(r, L)), v=synth.maxwell_velocities(n, 1.5, seed), L=L, n=n)
+
+
+@pytest.mark.parametrize("kind", ["fp64", "verlet", "tiles"])
+@pytest.mark.parametrize("n,cells", [(3000, 10), (3000, 11), (257, 24), (16384, 10), (16384, 32)])
+def test_sort_of_dilute_systems(pkg, oracle_mod, n, cells, kind):
+    """1,000 cells (the last sort within one cluster is at 1,024) and 1,331 to
+    32,768, most of them empty in the larger boxes: forces after steps with
+    rebuilds, at the GPU's own positions."""
+    s = dilute(n, cells, seed=cells)
+    kw = dict(fp64=dict(precision=pkg.MD_PREC_FP64), verlet=dict(precision=pkg.MD_PREC_MIXED),
+              tiles=dict(precision=pkg.MD_PREC_MIXED, pair_mode=pkg.MD_PAIR_TILES))[kind]
+    g = pkg.System(params(pkg, s, vacf=None, dt=0.02, **kw), s["r"], s["v"])
+    g.step(12)
+    got = g.particles()
+    assert g.observables()["rebuilds"] >= 2
+    g.close()
+    F, e, W = oracle_mod.lj_forces(got["r"], s["L"], method="cells")
+    if not F.any():  # the 257 atoms of the largest cells per atom: no pair in range
+        assert not got["F"].any()
+    elif kind == "fp64":
+        assert rel(got["F"], F) <= 1e-11
+        assert rel(got["W"], W) <= 1e-11
+    else:
+        check_mixed_forces(got["F"], F, got["r"], s["L"], oracle_mod)
+
+
+def test_dilute_sort_time_has_no_step_at_the_small_sort(pkg):
+    """16,384 atoms in 96^3 cells are on one side of the small sort's line by
+    atoms, 16,385 on the other: a step takes the same time on both (it took
+    four times as long below the line when cells did not count)."""
+    import time
+
+    best = []
+    for n in (16384, 16385):
+        s = dilute(n, 96, seed=3)
+        g = pkg.System(params(pkg, s, vacf=None, precision=pkg.MD_PREC_MIXED), s["r"], s["v"])
+        took = []
+        for _ in range(5):
+            t = time.perf_counter()
+            g.step(32)
+            g.observables()
+            took.append(time.perf_counter() - t)
+        best.append(min(took))
+        g.close()
+    assert best[0] <= 2.0 * best[1]
