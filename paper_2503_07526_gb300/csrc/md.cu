@@ -1504,10 +1504,24 @@ __device__ __forceinline__ float dist2(const float4 &a, const float4 &b) {
 // as blocks of eight in slot order, the last block of each segment padded with
 // the dummy slot 0.  A lane whose masks do not fit empties them on the way (all
 // lanes then do, in the same order of entries).
-constexpr int kFarWords = 24;  // far masks kept per thread (about 20 at a liquid's density)
-size_t build_smem(int wcap, int threads) {
-  return ((tile_smem(wcap, false) + 15) & ~(size_t)15) + (size_t)threads * kFarWords * 6;
+constexpr int kFarWords = 24;  // far masks kept per thread at most (about 20 at a liquid's density)
+// The masks lie over the window-cell bytes, which are read for the last time
+// when the window is staged, and a thread keeps as many as leave room for two
+// CTAs per SM (228 KB, of which each CTA loses 1 KB and the layout): 20 at the
+// largest window and CTA.  With 24 at any window, and beside the bytes, a CTA of
+// 384 threads had the SM to itself from 3,400 slots on: a step of a 256-replica
+// batch that rebuilds some replica on every step took 1,277 us with windows of
+// 3,648 slots and 1,094 with 4,096, now 1,070 and 950.
+constexpr int kBuildSmemMax = 228 * 1024 / 2 - 1024 - 128 - (int)sizeof(TileWin);
+__host__ __device__ constexpr int far_words(int wcap, int threads) {
+  const int fit = (kBuildSmemMax - (wcap + kWinPad) * (int)sizeof(float4)) / (threads * 6);
+  return fit < kFarWords ? fit : kFarWords;
 }
+constexpr size_t build_smem(int wcap, int threads) {
+  return (size_t)(wcap + kWinPad) * sizeof(float4) + (size_t)threads * far_words(wcap, threads) * 6;
+}
+static_assert(far_words(kWinMaxSlots, kTileThreadsMax) >= 16, "masks of the largest window and CTA");
+static_assert(128 * kFarWords * 6 >= kWinMaxSlots + kWinPad, "the masks hold the window-cell bytes of the smallest CTA");
 
 __global__ void __launch_bounds__(kTileThreadsMax, 2) k_build_tile(Sys d, LJ<float> lj) {
   if (!any_rebuild(d)) return;
@@ -1530,10 +1544,9 @@ __global__ void __launch_bounds__(kTileThreadsMax, 2) k_build_tile(Sys d, LJ<flo
   stage_coords<false>(d, W, whi, nullptr, cellof);
   const uint32_t wbase = (uint32_t)__cvta_generic_to_shared(whi);
   // this thread's far masks and their first slots, one row of the CTA each
-  uint32_t *fmask = reinterpret_cast<uint32_t *>(cellof + ((d.wcap + kWinPad + 15) & ~15)) + threadIdx.x;
-  unsigned short *fslot =
-      reinterpret_cast<unsigned short *>(fmask - threadIdx.x + kFarWords * blockDim.x) + threadIdx.x;
-  const int T = blockDim.x;
+  const int T = blockDim.x, words = far_words(d.wcap, T);
+  uint32_t *fmask = reinterpret_cast<uint32_t *>(cellof) + threadIdx.x;
+  unsigned short *fslot = reinterpret_cast<unsigned short *>(fmask - threadIdx.x + words * T) + threadIdx.x;
   const int64_t n = d.n;
   const int maxb = d.maxnb >> 3;
   int t1;
@@ -1616,7 +1629,7 @@ __global__ void __launch_bounds__(kTileThreadsMax, 2) k_build_tile(Sys d, LJ<flo
           }
         }
         if (fm) {
-          if (nw == kFarWords) {  // full: this lane empties its masks now
+          if (nw == words) {  // full: this lane empties its masks now
             for (uint32_t off = pop(); off; off = pop()) put_far(off);
             w = nw = kept = 0;
             early = true;
@@ -3183,7 +3196,7 @@ int finish_tiles(md_handle *h, cudaStream_t st) {
   OTF_CUDA(cudaMemcpyAsync(h->d_tiles, h->tiles_host.data(), nt * sizeof(Tile), cudaMemcpyHostToDevice, st));
   OTF_CUDA(cudaMemsetAsync(d.trec, 0xff, nt * sizeof(TileWin), st));
   OTF_CUDA(cudaFuncSetAttribute(k_build_tile, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)build_smem(kWinMaxSlots, kTileThreadsMax)));
+                                kBuildSmemMax));
   OTF_CUDA(cudaFuncSetAttribute(k_pair_tile, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)tile_smem(kWinMaxSlots, true)));
   return MD_OK;

@@ -244,3 +244,26 @@ def test_windows_of_unlike_size_in_one_process(pkg, use_graph):
         assert np.array_equal(got[key], want[key]), key
     other.close()
     g.close()
+
+
+@pytest.mark.parametrize("cells,rho,skin", [(25, 0.9, 0.5), (25, 0.8442, 0.3), (12, 0.9, 0.5)])
+def test_lists_do_not_depend_on_the_window_capacity(pkg, cells, rho, skin):
+    """A window of 4,096 slots leaves a CTA of 384 threads room for fewer far
+    masks per thread than a smaller one (20 instead of 24; about 27 are needed
+    at 28 atoms per cell), and a lane whose masks do not fit empties them on the
+    way: the same lists, so the same run bit for bit.  Every launch shape that
+    the autotuner tries is accepted with the largest window."""
+    s = jittered(cells, seed=3, rho=rho)
+    out = []
+    for slots in (0, 3648, 4096):
+        g = pkg.System(tiles(pkg, s, window_slots=slots, skin=skin, vacf=None, dt=0.02), s["r"], s["v"])
+        g.step(10)
+        assert g.observables()["rebuilds"] >= 2
+        out.append(g.particles())
+        if cells == 25 and skin == 0.5:
+            assert g.config()["tile_threads"] == 384
+        g.close()
+    for got in out[1:]:
+        for key in ("r", "v", "F", "W", "epot"):
+            assert np.array_equal(got[key], out[0][key]), key
+    pkg.System(tiles(pkg, s, window_slots=4096, skin=skin, vacf=None, autotune=True), s["r"], s["v"]).step(2)
