@@ -777,12 +777,15 @@ struct AdamStep {
   float lr, beta1, beta2, eps, wd, c1, c2;
 };
 // One parameter's step; decay: the weight decay of this parameter (0: a bias).
+// Every rounding is written out: left to the compiler, k_adam and
+// k_train_cluster contracted the moments differently, and an ulp of a weight
+// can turn its bfloat16 rounding.
 __device__ __forceinline__ float adam_one(const AdamStep &k, float w, float g, float &m1, float &m2, bool decay) {
-  m1 = k.beta1 * m1 + (1.f - k.beta1) * g;
-  m2 = k.beta2 * m2 + (1.f - k.beta2) * g * g;
-  float step = (m1 / k.c1) / (sqrtf(m2 / k.c2) + k.eps);
-  if (decay) step += k.wd * w;
-  return w - k.lr * step;
+  m1 = __fmaf_rn(1.f - k.beta1, g, __fmul_rn(k.beta1, m1));
+  m2 = __fmaf_rn(__fmul_rn(1.f - k.beta2, g), g, __fmul_rn(k.beta2, m2));
+  float step = __fdiv_rn(__fdiv_rn(m1, k.c1), __fadd_rn(__fsqrt_rn(__fdiv_rn(m2, k.c2)), k.eps));
+  if (decay) step = __fmaf_rn(k.wd, w, step);
+  return __fmaf_rn(-k.lr, step, w);
 }
 __global__ void k_adam(float *__restrict__ w, const float *__restrict__ g, float *__restrict__ m1,
                        float *__restrict__ m2, int64_t count, AdamTable tab, AdamStep k) {

@@ -300,3 +300,39 @@ def test_training_stops_at_the_first_epoch_that_gives_up(pkg):
         got.append(net.get_flat())
         net.close()
     assert np.array_equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("n_in,depth,batch,batches", [(132, 3, 128, 3), (20, 1, 128, 2), (240, 2, 256, 2), (64, 6, 384, 2),
+                                                      (132, 3, 1152, 1)])
+def test_training_equals_layered_steps_bit_for_bit(pkg, n_in, depth, batch, batches):
+    """Two calls of mlp_train (two epochs, then one), an Adam step on the
+    gradients that the last batch left, and a layered step: weights and
+    gradients equal those of the same steps through mlp_loss_grad and
+    mlp_adam_step bit for bit, so the moments, the step count and the kept
+    gradients pass between the two paths as they are."""
+    rows = batch * batches
+    X = synth.normal(75, rows * n_in).reshape(rows, n_in).astype(np.float32)
+    T = synth.normal(76, rows * 2).reshape(rows, 2).astype(np.float32)
+    start = f32(synth.mlp_init(77, (n_in,) + (128,) * depth + (2,), bias_scale=0.1))
+    order = synth.permutations(78, 3, rows)
+    kw = dict(depth=depth, batch=batch, lr=1e-3, weight_decay=1e-3)
+    a, b = pkg.MLP(n_in, 2, **kw), pkg.MLP(n_in, 2, **kw)
+    a.set_params(start)
+    b.set_params(start)
+    a.train(X, T, 2, order=order[:2])
+    a.train(X, T, 1, order=order[2:])
+    for e in range(3):
+        for k in range(batches):
+            at = order[e, k * batch:(k + 1) * batch]
+            b.loss_grad(X[at], T[at])
+            b.adam_step()
+    assert np.array_equal(a.get_flat(), b.get_flat())
+    a.adam_step()
+    b.adam_step()
+    assert np.array_equal(a.get_flat(), b.get_flat())
+    la, ga = a.loss_grad(X[:batch], T[:batch])
+    lb, gb = b.loss_grad(X[:batch], T[:batch])
+    a.adam_step()
+    b.adam_step()
+    assert la == lb and np.array_equal(ga, gb)
+    assert np.array_equal(a.get_flat(), b.get_flat())
