@@ -192,3 +192,38 @@ def test_ionic_rejects_bad_setups(pkg, system):
     with pytest.raises(pkg.MdError):  # replicas are Lennard-Jones only
         reps = [dict(r=s["r"], v=s["v"], box=s["L"], types=s["types"])] * 2
         pkg.System(params(pkg, s, 1), replicas=reps)
+
+
+def test_fp64_pair_terms_are_accurate_to_their_last_bits(pkg):
+    """Uncharged dimers 8 to 10 A apart, each alone, on coordinates whose
+    differences and squares are exact (cells of 16 A, multiples of 2^-20):
+    A exp(-r / rho) with rho = 1 / 16 magnifies an error of r (half a unit of
+    2^-49 when rounded correctly) 16 times.  Beyond that: three units of 2^-52
+    for the exponential, the product and the sum, five more for the force."""
+    from decimal import Decimal, getcontext
+
+    getcontext().prec = 40
+    corner = np.stack(np.meshgrid(*[[6.0, 38.0]] * 3, indexing="ij")).reshape(3, 8)
+    eps, worst = 2.0 ** -52, [0.0, 0.0]
+    for k in range(25):
+        u = synth.uniform01(500 + k, 32).reshape(4, 8)
+        d = u[:3] - 0.5
+        d = np.round(d / np.sqrt((d ** 2).sum(0)) * (8.02 + 1.96 * u[3]) * 2 ** 20) / 2 ** 20
+        at = corner + np.round(u[:3] * 2 ** 20) / 2 ** 20
+        r = np.mod(np.concatenate([at, at + d], axis=1), 64.0)
+        p = pkg.make_params(16, 64.0, rc=10.0, dt=0.05, skin=6.0, precision=pkg.MD_PREC_FP64, masses=(20.0,),
+                            potential=pkg.MD_POT_BUCK_EWALD, charges=(0.0,), buckingham=(1200.0, 0.0625, 0.0),
+                            ewald_alpha=0.3, mesh=16, order=8, stress=(4, 16, 2, 1), heatflux=(4, 16, 2, 1), vacf=None)
+        g = pkg.System(p, r, np.zeros((3, 16)))
+        got = g.particles()
+        g.close()
+        for q in range(8):
+            dist = sum(Decimal(float(x)) ** 2 for x in d[:, q]).sqrt()
+            e = 600 * (-16 * dist).exp()  # half of the pair's energy
+            a = int(np.abs(d[:, q]).argmax())
+            f = 2 * e * 16 / dist * Decimal(float(d[a, q]))  # on the second ion
+            worst[0] = max(worst[0], abs(float((Decimal(float(got["epot"][q])) - e) / e)))
+            worst[1] = max(worst[1], abs(float((Decimal(float(got["F"][a, 8 + q])) - f) / f)))
+    print(f"energy {worst[0]:.3e} force {worst[1]:.3e}")
+    assert worst[0] <= 16 * 2.0 ** -50 + 3 * eps
+    assert worst[1] <= 16 * 2.0 ** -50 + 8 * eps
