@@ -6,9 +6,9 @@ per-step observables (stress tensor and heat flux, Sec. 2.3) built from them.
 System: 1,728 ions (rock salt 6^3 x 8 at 0.031 ions / A^3, L = 38.2 A, every
 ion displaced by up to 0.3 A), charges +1 / -1 e, Na / Cl masses, Buckingham
 A = 1200 eV, rho = 0.32 A, C = 10 eV A^6 for every pair, rc = 10 A, Ewald
-alpha = 0.3 / A, order-8 splines on a 16^3 mesh (the chunks of a cell row fit
-the kernels' shared tiles) and on a 32^3 mesh (they do not: the kernels take
-the global mesh directly); units eV, A, amu, e.
+alpha = 0.3 / A, order-8 splines on a 16^3 mesh and on a 32^3 mesh (the chunks
+of a cell row fit the kernels' shared tiles on both; test_gpu_sizes.py has a
+mesh too fine for them); units eV, A, amu, e.
 
 Tolerances.  FP64: the charge mesh is summed in 128-bit fixed point with
 2^-80 resolution per contribution (so that the sums do not depend on the

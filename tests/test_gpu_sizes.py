@@ -141,6 +141,64 @@ def test_ionic_sizes_and_orders_match_oracle(pkg, system, precision, copies, ord
         assert rel(got[key], want) <= t, key
 
 
+def chunk_volumes(r, L, mesh, order, chunk=32):
+    """Mesh points of the box that each 32 consecutive ions of a cell row reach,
+    in the order of the sort (cells of rc + skin = 11 A, x fastest, then octant
+    and number)."""
+    nc = int(L // 11.0)
+    e = L / nc
+    c = np.minimum((r / e).astype(int), nc - 1)
+    octant = ((r >= (c + 0.5) * e) * np.array([[1], [2], [4]])).sum(0)
+    row = c[2] * nc + c[1]
+    at = np.lexsort((np.arange(r.shape[1]), octant, c[0], row))
+    u = np.floor(r * (mesh / L)).astype(int)
+    out = []
+    for k in range(nc * nc):
+        mine = at[row[at] == k]
+        for a in range(0, len(mine), chunk):
+            x = u[:, mine[a:a + chunk]]
+            out.append(np.prod(x.max(1) - x.min(1) + order))
+    return np.array(out)
+
+
+@pytest.mark.parametrize("order", [4, 6, 8])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_ionic_meshes_too_fine_for_the_tiles(pkg, system, precision, order):  # noqa: F811
+    """192 mesh points over three cells: every chunk reaches more points than the
+    largest shared tile of the spread (160 KB, a value a point) and of the gather
+    (two) holds, so charges go straight to the global mesh and are read from
+    there: forces, energies and virials against the oracle, and two runs bit for
+    bit.  The mixed form's virials carry the FP32 rounding of the mesh times
+    second derivatives of the weights, that is (K / L)^2: the bound of the tests
+    with 32 points times (K / 32)^2."""
+    from oracle import ewald
+
+    s, K = system, 192
+    r = np.mod(s["r"], s["L"])
+    assert chunk_volumes(r, s["L"], K, order).min() > 160 * 1024 / 4
+    if (K, order) not in _MESH:
+        q = np.where(s["types"] == 0, 1.0, -1.0)
+        base = reference(s, 16)  # real-space and self terms; its mesh terms are exchanged
+        F8, E8, W8, _, _ = ewald.spme_reciprocal(r, q, s["L"], alpha=ALPHA, K=16, order=8)
+        Fk, Ek, Wk, _, _ = ewald.spme_reciprocal(r, q, s["L"], alpha=ALPHA, K=K, order=order)
+        _MESH[K, order] = dict(F=base["F"] - F8 + Fk, epot=base["epot"] - E8 + Ek, W=base["W"] - W8 + Wk)
+    want = _MESH[K, order]
+    p = ionic_params(pkg, s, precision, mesh=K)
+    p.order = order
+    after = []
+    for _ in range(2):
+        g = pkg.System(p, s["r"], s["v"], types=s["types"])
+        got = g.particles()
+        for key, t in (("F", 1e-11 if precision == 0 else 2e-5), ("epot", 1e-11 if precision == 0 else 1e-4),
+                       ("W", 1e-11 if precision == 0 else 1e-4 * (K / 32) ** 2)):
+            assert rel(got[key], want[key]) <= t, key
+        g.step(5)
+        after.append(g.particles())
+        g.close()
+    for key in ("r", "v", "F", "W", "epot"):
+        assert np.array_equal(after[0][key], after[1][key]), key
+
+
 @pytest.mark.parametrize("b,p,m,ns,gs,prec,S", [
     (4, 16, 2, 4864, 2432, 0, 100), (4, 16, 2, 4865, 973, 0, 100), (3, 32, 2, 4864, 1216, 1, 90),
     (3, 32, 4, 4866, 811, 1, 90), (2, 16, 2, 300002, 150001, 1, 40), (2, 16, 2, 600000, 200000, 1, 40),
