@@ -488,8 +488,11 @@ int launch_grouped_block(const CorrDev &c, const Tin *x, BlockIdx bi, cudaStream
 
 template <typename T, typename Tin>
 int launch_series(const CorrDev &c, const Tin *x, const Tin *y, PushIdx pi, cudaStream_t s) {
-  // a warp per series while those warps fit the GPU at once (32 per SM)
-  if (c.ns <= 152 * 32) {
+  // a warp per series while those warps fit the GPU at once (32 per SM); with at
+  // most four lags most of a warp's lanes idle and, in FP64, the thread's serial
+  // walk is the faster one from some 2,000 series on (4,864 series of two lags:
+  // 7.5 us by warps, 5.7 by threads; of four 7.5 and 6.0; of six 7.5 and 8.0)
+  if (c.ns <= 152 * (sizeof(T) == 8 && c.p <= 4 ? 8 : 32)) {
     k_push_series_warp<T, Tin><<<ceil_div(c.ns * kWarp, 128), 128, 0, s>>>(c, x, y, pi);
     OTF_LAUNCH_CHECK();
     return MD_OK;

@@ -269,3 +269,49 @@ def test_dilute_sort_time_has_no_step_at_the_small_sort(pkg):
         best.append(min(took))
         g.close()
     assert best[0] <= 2.0 * best[1]
+
+
+@pytest.mark.parametrize("p,m,ns", [(2, 2, 1216), (2, 2, 1217), (4, 2, 1216), (4, 2, 1217), (4, 4, 4864), (4, 2, 4865),
+                                    (6, 2, 4864)])
+@pytest.mark.parametrize("cross", [False, True])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_corr_push_of_few_lags(pkg, oracle_mod, p, m, ns, cross, prec):
+    """Up to four lags a warp per series ends at 1,216 series in FP64, else at
+    4,864."""
+    x, y = series(ns, 70, seed=ns + p), series(ns, 70, seed=ns + p + 1)
+    g = pkg.Corr.create(4, p, m, ns, cross=cross, precision=prec)
+    o = oracle_mod.Corr(4, p, m, ns, 1, cross)
+    for t in range(70):
+        g.push(x[t], y[t] if cross else None)
+        o.push(x[t], y[t] if cross else None)
+    gv, gc, gu = g.raw()
+    ov, oc, ou = o.raw()
+    assert gu == ou and np.array_equal(gc, oc)
+    gv, ov = np.reshape(gv, -1), np.reshape(ov, -1)
+    assert np.abs(gv - ov).max() <= (1e-11 if prec == 0 else 2e-5) * np.abs(ov).max()
+    g.close()
+
+
+def test_push_time_of_few_lags_has_no_step_at_the_warps_line(pkg):
+    """FP64 correlators of two lags with 4,864 and 4,865 series take the same
+    time a push (7.5 and 5.7 us where the warps went on to 4,864 at any number
+    of lags)."""
+    import time
+
+    import torch
+
+    best = []
+    for ns in (4864, 4865):
+        g = pkg.Corr.create(4, 2, 2, ns, precision=0)
+        rows = list(torch.randn(256, ns, device="cuda", dtype=torch.float64))
+        took = []
+        for _ in range(12):
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            for row in rows:
+                g.push(row)
+            torch.cuda.synchronize()
+            took.append(time.perf_counter() - t)
+        best.append(min(took))
+        g.close()
+    assert best[0] <= 1.15 * best[1]
