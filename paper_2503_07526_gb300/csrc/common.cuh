@@ -104,16 +104,16 @@ struct dfloat {
   float h, l;
 };
 
-__host__ __device__ __forceinline__ dfloat df_fast_two_sum(float a, float b) {  // needs |a| >= |b|
+__device__ __forceinline__ dfloat df_fast_two_sum(float a, float b) {  // needs |a| >= |b|
   const float s = a + b;
   return dfloat{s, b - (s - a)};
 }
-__host__ __device__ __forceinline__ dfloat df_two_sum(float a, float b) {
+__device__ __forceinline__ dfloat df_two_sum(float a, float b) {
   const float s = a + b;
   const float bb = s - a;
   return dfloat{s, (a - (s - bb)) + (b - bb)};
 }
-__host__ __device__ __forceinline__ dfloat df_add(dfloat a, dfloat b) {
+__device__ __forceinline__ dfloat df_add(dfloat a, dfloat b) {
   dfloat s = df_two_sum(a.h, b.h);
   const dfloat t = df_two_sum(a.l, b.l);
   s.l += t.h;
@@ -121,7 +121,7 @@ __host__ __device__ __forceinline__ dfloat df_add(dfloat a, dfloat b) {
   s.l += t.l;
   return df_fast_two_sum(s.h, s.l);
 }
-__host__ __device__ __forceinline__ dfloat df_mul(dfloat a, dfloat b) {
+__device__ __forceinline__ dfloat df_mul(dfloat a, dfloat b) {
   const float p = a.h * b.h;
   float e = fmaf(a.h, b.h, -p);
   e = fmaf(a.h, b.l, e);
@@ -206,26 +206,6 @@ __device__ __forceinline__ void warp_sum16(dfacc (&a)[16]) {
   const float s2 = __shfl_xor_sync(0xffffffffu, a[0].s, 1);
   const float c2 = __shfl_xor_sync(0xffffffffu, a[0].c, 1);
   a[0].merge(s2, c2);
-}
-
-// The mesh coordinate num / den + off kl (a cell centre's, an exact fraction, and
-// an offset from it) as its integer part and its fraction rounded to FP32 once:
-// the integer comes off the high word with its rounding error kept, which a
-// small negative coordinate has (rounded there and again with the low word, one
-// fraction in eighty was off by up to 0.75 of an ulp).
-__host__ __device__ __forceinline__ float df_fraction(int num, int den, dfloat off, dfloat kl, int &base) {
-  const int q = num / den;
-  const float fd = (float)den, rem = (float)(num - q * den), h = rem / fd;
-  const dfloat u = df_add(dfloat{h, fmaf(-h, fd, rem) / fd}, df_mul(off, kl));
-  float fl = floorf(u.h);
-  const dfloat d = df_two_sum(u.h, -fl);
-  float f = d.h + (d.l + u.l);
-  if (f < 0.f) {
-    f += 1.f;
-    fl -= 1.f;
-  }
-  base = q + (int)fl;
-  return f;
 }
 
 // Host / FP64 conversions (used at set-up and output only).

@@ -121,9 +121,22 @@ __device__ __forceinline__ void mesh_coords(const SpmeAtoms &a, int64_t i, const
   } else {
     const float4 l4 = a.rlo[i];
     const float oh[3] = {r.x, r.y, r.z}, ol[3] = {l4.x, l4.y, l4.z};
+    const int den = 2 * a.nc;
+    const float fd = (float)den;
 #pragma unroll
-    for (int ax = 0; ax < 3; ++ax)
-      frac[ax] = df_fraction((2 * cc[ax] + 1) * g.K, 2 * a.nc, dfloat{oh[ax], ol[ax]}, dfloat{g.kl_h, g.kl_l}, base[ax]);
+    for (int ax = 0; ax < 3; ++ax) {
+      const int num = (2 * cc[ax] + 1) * g.K, q = num / den;
+      const float rem = (float)(num - q * den);  // below 2^11: exact
+      const float h = rem / fd;
+      const dfloat u = df_add(dfloat{h, fmaf(-h, fd, rem) / fd}, df_mul(dfloat{oh[ax], ol[ax]}, dfloat{g.kl_h, g.kl_l}));
+      float fl = floorf(u.h), f = (u.h - fl) + u.l;
+      if (f < 0.f) {
+        f += 1.f;
+        fl -= 1.f;
+      }
+      base[ax] = q + (int)fl;
+      frac[ax] = f;
+    }
   }
 #pragma unroll
   for (int ax = 0; ax < 3; ++ax) base[ax] = max(-g.K, min(2 * g.K, base[ax]));
