@@ -100,10 +100,12 @@ struct MeshPlan {
 // within a box of the box, so that a non-finite coordinate (which md_step
 // reports) cannot index anything.
 //
-// Mixed form: in double-float arithmetic (~48 bits, rounded to FP32 once, like
-// the FP64 arithmetic of the other form): the cell centre in mesh units is
-// (2 c + 1) K / (2 nc), split exactly into integer and fraction.  Its ~36 FP64
-// operations per atom took 33 us of each kernel at 512,000 ions.
+// Mixed form: in double-float arithmetic (~48 bits) instead of FP64: the cell
+// centre in mesh units is (2 c + 1) K / (2 nc), split exactly into integer and
+// fraction.  The fraction is rounded to FP32 once, as from FP64, except where the
+// coordinate is a small negative number, whose high word is rounded when its
+// floor comes off (errors 1.33e-8 rms and 4.5e-8 at most, from FP64 1.30e-8 and
+// 3.0e-8).  The ~36 FP64 operations per atom took 33 us of each kernel at 512,000 ions.
 template <typename T>
 __device__ __forceinline__ void mesh_coords(const SpmeAtoms &a, int64_t i, const MeshPlan &g,
                                             const typename Rec<T>::type &r, int (&base)[3], T (&frac)[3]) {
@@ -356,8 +358,8 @@ struct SpreadPitch {
 // Against a thread per mesh column that tests every atom of the chunk (a third
 // of the tests hit, and its flush walked z in each thread): 440 -> 156 us at
 // 512,000 ions (mixed form, 128^3 mesh, order 8), 410 -> 35 us at 1,728 (FP64,
-// 32^3).  What is left is issue (62 %): ~260 warp instructions per atom, half
-// of them the tile additions, a fifth the flush.
+// 32^3).  What is left is the load/store unit (77 %; issue 72 %, mixed form): 256
+// warp instructions per atom, half of them the tile additions, a fifth the flush.
 template <typename T, int N>
 __global__ void __launch_bounds__(kRowThreads) k_spme_spread(SpmeAtoms a, MeshPlan g, unsigned long long *Qi) {
   using R = typename Rec<T>::type;
@@ -637,7 +639,8 @@ __device__ __forceinline__ void gather_lane(const T *w, int z, Pair<T> mid, Fetc
 // lanes sum the points of one atom each (gather_lane: 5 operations per point
 // where the separate ten sums took 14, and 64-byte rows of the tile where a
 // thread per atom read 32 unrelated places per load).  At 512,000 ions in the
-// mixed form, order 8: 297 -> 220 us; at 1,728 ions in FP64 319 -> 44 us.
+// mixed form, order 8: 297 -> 220 us; at 1,728 ions in FP64 319 -> 44 us.  Bound
+// by the shared-memory pipe (81 %, a third of its wavefronts conflict replays).
 template <typename T, int N>
 __global__ void __launch_bounds__(kRowThreads, sizeof(T) == 4 ? 5 : 2)
     k_spme_gather(SpmeAtoms a, MeshPlan g, const T *phi, const T *psi, T ke, T kL, T cw, T self, T *F, T *epot, T *W) {
